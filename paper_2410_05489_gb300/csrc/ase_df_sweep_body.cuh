@@ -230,6 +230,20 @@ struct Tile {
   static constexpr size_t smem_doubles = queue_offset + ((size_t)QCAP + 2 + 1) / 2;
 };
 
+// Quotient and remainder by a tile's run-time line count n (at most 127) of an index below 2^13, by
+// a multiplication: with m = ceil(2^20 / n), i m / 2^20 exceeds i / n by less than 2^13 / 2^20 <
+// 1 / n.  An integer division by a run-time number costs some 25 instructions, and the staging
+// and item loops do one per element.
+struct LineDiv {
+  unsigned int m;
+  int n;
+  __device__ __forceinline__ explicit LineDiv(int n_) : m(((1u << 20) + n_ - 1) / n_), n(n_) {}
+  __device__ __forceinline__ void split(int i, int& q, int& r) const {
+    q = (int)(((unsigned int)i * m) >> 20);
+    r = i - q * n;
+  }
+};
+
 // Deferral of the work items whose branch is the WENOZ-AO(5,3)+DF fallback.  Its arithmetic
 // (smoothness indicators, nonlinear weights, four sub-polynomials) is several times that of
 // a linear branch, so a warp holding one such item among linear ones would run the long path
@@ -282,32 +296,54 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   int* s_queue = reinterpret_cast<int*>(smem + TL::queue_offset);
   unsigned int* s_qn = reinterpret_cast<unsigned int*>(s_queue + TL::QCAP);
   if (tid < 2) s_qn[tid] = 0u;
-  // ---- stage cell averages: cells a0-1-K .. a0+TN-1+K, lines b0-KT .. b0+tt+KT-1 ----
-  for (int idx = tid; idx < C * nb * NA; idx += NT) {
-    int c, bb, aa;
-    if (DIR == 0) { aa = idx % NA; bb = (idx / NA) % nb; c = idx / (NA * nb); }
-    else { bb = idx % nb; aa = (idx / nb) % NA; c = idx / (NA * nb); }
+  // ---- staging: consecutive threads take consecutive addresses along the direction in which the
+  // arrays are contiguous (the sweep for x-faces, the lines for y-faces) ----
+  static_assert(NA * NB < (1 << 13) && NB < 128, "LineDiv range");
+  const LineDiv dnb(nb);
+  const int sta = (DIR == 0) ? 1 : g.nx, stb = (DIR == 0) ? g.nx : 1;
+  // a tile whose halo lies inside the grid needs none of the boundary's index maps
+  const bool inside = DIM == 2 && a0 - 1 - K >= 0 && a0 + TN - 1 + K < n && b0 - KT >= 0 && b0 + tt + KT <= mlin;
+  // cell averages: cells a0-1-K .. a0+TN-1+K, lines b0-KT .. b0+tt+KT-1
+  for (int idx = tid; idx < nb * NA; idx += NT) {
+    int bb, aa;
+    if (DIR == 0) { aa = idx % NA; bb = idx / NA; }
+    else dnb.split(idx, aa, bb);
     const int a = a0 - 1 - K + aa, b = b0 - KT + bb;
-    const int i = (DIR == 0) ? a : b, j = (DIR == 0) ? b : a;
-    sW[(c * NB + bb) * NA + aa] = fetch_w(g, args.W, c, i, j, ts);
+    double* dst = sW + bb * NA + aa;
+    if (inside) {
+      const double* src = args.W + (size_t)b * stb + (size_t)a * sta;
+#pragma unroll
+      for (int c = 0; c < C; ++c) dst[c * NB * NA] = __ldg(src + (size_t)c * g.nx * g.ny);
+    } else {
+      const int i = (DIR == 0) ? a : b, j = (DIR == 0) ? b : a;
+#pragma unroll 1
+      for (int c = 0; c < C; ++c) dst[c * NB * NA] = fetch_w(g, args.W, c, i, j, ts);
+    }
   }
-  // ---- normal face strengths: faces a0-K .. a0+TN-1+K of every staged line ----
+  // normal face strengths: faces a0-K .. a0+TN-1+K of every staged line
   for (int idx = tid; idx < nb * NSN; idx += NT) {
     int fa, bb;
     if (DIR == 0) { fa = idx % NSN; bb = idx / NSN; }
-    else { bb = idx % nb; fa = idx / nb; }
-    sSn[bb * NSN + fa] = (DIR == 0) ? sigma_x_at(g, args.s_norm, a0 - K + fa, b0 - KT + bb)
-                                    : sigma_y_at(g, args.s_norm, a0 - K + fa, b0 - KT + bb);
+    else dnb.split(idx, fa, bb);
+    const int f = a0 - K + fa, b = b0 - KT + bb;
+    double v;
+    if (inside) v = __ldg(args.s_norm + ((DIR == 0) ? (size_t)b * (g.nx + 1) + f : (size_t)f * g.nx + b));
+    else v = (DIR == 0) ? sigma_x_at(g, args.s_norm, f, b) : sigma_y_at(g, args.s_norm, f, b);
+    sSn[bb * NSN + fa] = v;
   }
-  // ---- tangential face strengths of the reconstructing cells' columns ----
+  // tangential face strengths of the reconstructing cells' columns: faces b0-K+1 .. b0+tt+K-1
   if (DIM == 2) {
-    const int nst = tt + 2 * K - 1;  // tangential faces b0-K+1 .. b0+tt+K-1
+    const int nst = tt + 2 * K - 1;
+    const LineDiv dst(nst);
     for (int idx = tid; idx < NQ * nst; idx += NT) {
       int qa, fb;
       if (DIR == 0) { qa = idx % NQ; fb = idx / NQ; }
-      else { fb = idx % nst; qa = idx / nst; }
-      sSt[qa * NST + fb] = (DIR == 0) ? sigma_y_at(g, args.s_tan, b0 - K + 1 + fb, a0 - 1 + qa)
-                                      : sigma_x_at(g, args.s_tan, b0 - K + 1 + fb, a0 - 1 + qa);
+      else dst.split(idx, qa, fb);
+      const int f = b0 - K + 1 + fb, a = a0 - 1 + qa;
+      double v;
+      if (inside) v = __ldg(args.s_tan + ((DIR == 0) ? (size_t)f * g.nx + a : (size_t)a * (g.nx + 1) + f));
+      else v = (DIR == 0) ? sigma_y_at(g, args.s_tan, f, a) : sigma_x_at(g, args.s_tan, f, a);
+      sSt[qa * NST + fb] = v;
     }
   }
   __syncthreads();
@@ -326,12 +362,10 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       int qa, bb, pt;  // pt -1: an interior cell, both points; 0 / 1: an end cell, one point
       if (it < (NQ - 2) * nb) {
         if (DIR == 0) { qa = 1 + it % (NQ - 2); bb = it / (NQ - 2); }
-        else { bb = it % nb; qa = 1 + it / nb; }
+        else { dnb.split(it, qa, bb); ++qa; }
         pt = -1;
       } else {
-        const int e = it - (NQ - 2) * nb;
-        bb = e % nb;  // pt 0: cell qa = 0 at xi = 0; 1: qa = NQ-1 at xi = -1
-        pt = e / nb;
+        dnb.split(it - (NQ - 2) * nb, pt, bb);  // pt 0: cell qa = 0 at xi = 0; 1: qa = NQ-1 at xi = -1
         qa = pt * (NQ - 1);
       }
       const Branch br = select_branch<R>(sSn + bb * NSN + qa, g.thres);
@@ -362,6 +396,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
 
   // ---- phase 2: faces ----
   // Faces with a fallback tangential reconstruction on either side are deferred (2D).
+  const LineDiv dtt(tt);
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
     const int count = (pass == 0) ? TN * tt : (int)s_qn[1];
@@ -369,7 +404,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       const int it = (pass == 0) ? k : s_queue[k];
       int fa, tb;
       if (DIR == 0) { fa = it % TN; tb = it / TN; }
-      else { tb = it % tt; fa = it / tt; }
+      else dtt.split(it, fa, tb);
       const int f = a0 + fa, b = b0 + tb;
       if (f > n || b >= mlin) continue;
       Branch bt[2];
