@@ -99,6 +99,18 @@ template <int DIM>
 __global__ void __launch_bounds__(256) max_speed_kernel(const GridInfo g, const SpeedArgs a) {
   const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
   max_speed_range<DIM>(g, a, first, (size_t)g.nx * g.ny, stride);
+  if (DIM == 2 && a.sx != nullptr) {
+    front_range(a.sx, first, (size_t)g.ny * (g.nx + 1), stride, g.thres, &a.st->front[0]);
+    front_range(a.sy, first, (size_t)(g.ny + 1) * g.nx, stride, g.thres, &a.st->front[0]);
+  }
+}
+
+__global__ void __launch_bounds__(256) strength_kernel(const double* __restrict__ sx, size_t nsx,
+                                                       const double* __restrict__ sy, size_t nsy, double thres,
+                                                       DevState* st) {
+  const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+  front_range(sx, first, nsx, stride, thres, &st->front[0]);
+  front_range(sy, first, nsy, stride, thres, &st->front[0]);
 }
 
 __global__ void state_kernel(DevState* st, int op, double t) {
@@ -112,6 +124,7 @@ __global__ void state_kernel(DevState* st, int op, double t) {
     st->frozen_total = 0ull;
     st->bar_count = 0u;
     st->bar_gen = 0u;
+    for (int k = 0; k < 3; ++k) st->front[k] = 0u;
   } else if (op == 2) {  // the barrier's arrivals after a barrier that gave up
     st->bar_count = 0u;
   }
@@ -199,6 +212,12 @@ cudaError_t launch_max_speed(int dim, const GridInfo& g, const SpeedArgs& a, cud
   const int nt = cell_block(ncell);
   if (dim == 1) max_speed_kernel<1><<<grid_for(ncell, nt), nt, 0, s>>>(g, a);
   else max_speed_kernel<2><<<grid_for(ncell, nt), nt, 0, s>>>(g, a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_strength(const GridInfo& g, const double* sx, const double* sy, DevState* st, cudaStream_t s) {
+  const size_t nsx = (size_t)g.ny * (g.nx + 1), nsy = (size_t)(g.ny + 1) * g.nx;
+  strength_kernel<<<grid_for(nsx, 256), 256, 0, s>>>(sx, nsx, sy, nsy, g.thres, st);
   return cudaGetLastError();
 }
 

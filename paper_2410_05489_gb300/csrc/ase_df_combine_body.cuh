@@ -109,6 +109,7 @@ __device__ __forceinline__ void combine_range(const GridInfo& g, const CombineAr
     atomicAdd(&a.st->cnt[0], nmarked);
     atomicAdd(&a.st->repaired_total, (unsigned long long)nmarked);
   }
+  if (leader && DIM == 2) a.st->front[a.stage > 0 ? a.stage - 1 : 0] = 0u;  // the stage's sweeps have read it
   if (a.stage == 3 && leader) {
     a.st->t += dt;
     a.st->last_dt = dt;
@@ -153,6 +154,7 @@ __device__ __forceinline__ void repair_range(const GridInfo& g, const RepairArgs
       fU = self || (ju >= 0 && marked(i, ju));
     }
     if (!(fL || fR || fD || fU)) continue;
+    if (DIM == 2 && a.front_out != nullptr) *a.front_out = 1u;  // strengths of kSigmaBig
     double F[2][2][C];  // [dir][lower / upper face][component]
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
@@ -283,6 +285,15 @@ __device__ __forceinline__ void max_speed_range(const GridInfo& g, const SpeedAr
   if ((threadIdx.x & 31) == 0 && smax > 0.0)
     atomicMax(&a.st->max_speed_bits, (unsigned long long)__double_as_longlong(smax));
   if (bad) atomicOr(&a.st->flags, 0x1u);
+}
+
+// Raises *front when one of entries first, first + stride, ... < n of s is a front.
+__device__ __forceinline__ void front_range(const double* __restrict__ s, size_t first, size_t n, size_t stride,
+                                            double thres, unsigned int* front) {
+  const unsigned long long lim = smooth_limit(thres);
+  bool any = false;
+  for (size_t k = first; k < n; k += stride) any |= is_front(s[k], lim);
+  if (any) *front = 1u;
 }
 
 }  // namespace

@@ -33,6 +33,16 @@ __device__ __forceinline__ bool pos_finite(double x) {
 // Equals (a < t) except for a NaN with the sign bit set.
 __device__ __forceinline__ bool lt_pos(double a, double t) { return dbits(a) < dbits(t); }
 
+// Strengths up to this bit pattern (thres / 16) make every stencil sum of at most 8 of them smooth
+// (select_branch); a strength beyond it, or a negative or NaN one, is a front.
+__device__ __forceinline__ unsigned long long smooth_limit(double thres) {
+  const long long tb = dbits(thres);
+  return ((tb >> 52) > 4) ? (unsigned long long)(tb - (4LL << 52)) : 0ull;
+}
+__device__ __forceinline__ bool is_front(double s, unsigned long long limit) {
+  return (unsigned long long)dbits(s) > limit;
+}
+
 // max of two non-negative values, by bit pattern
 __device__ __forceinline__ double max_nonneg(double a, double b) { return dbits(a) < dbits(b) ? b : a; }
 

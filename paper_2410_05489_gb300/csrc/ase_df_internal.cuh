@@ -104,6 +104,11 @@ struct DevState {
   // Grid barrier of the single-launch repair (repair_all_kernel): arrivals and generation.
   // bar_count is 0 between barriers; ase_df_reset clears both.
   unsigned int bar_count, bar_gen;
+  // front[s]: the strengths that stage s + 1 (or a residual: s = 0) of a 2D problem consumes hold
+  // a front (is_front); raised by the kernel that reads the caller's strengths before the first
+  // stage and by each stage's sweeps and repair for the next, lowered by the consuming stage's
+  // combine.
+  unsigned int front[3];
 };
 
 // Slots of the branch histogram: linear 9th, 7th, 5th order, WENOZ-AO(5,3)+DF, linear 3rd
@@ -138,6 +143,8 @@ struct SweepArgs {
   double* s_out;          // sigma_out of this direction
   DevState* st;
   double tfrac = 0.0;     // the stage's time is st->t + tfrac st->dt (time-dependent ghosts)
+  const unsigned int* front = nullptr;  // whether s_norm, s_tan hold a front (2D; nullptr: no)
+  unsigned int* front_out = nullptr;    // raised when s_out does (or nullptr)
   unsigned long long* hist = nullptr;  // branch histogram (kBranchSlots counters) or nullptr
 };
 
@@ -170,12 +177,15 @@ struct RepairArgs {
   int stage;
   int pass;           // 1..kRepairPasses
   double tfrac = 0.0; // the stage's time is st->t + tfrac dt (time-dependent ghosts)
+  unsigned int* front_out = nullptr;  // raised with the strengths of first-order faces (2D)
 };
 
 struct SpeedArgs {
   const double* W;
   DevState* st;
   double inv_dx, inv_dy;
+  // 2D: the strengths of the same state, looked through for a front (nullptr: not looked for)
+  const double *sx = nullptr, *sy = nullptr;
 };
 
 // Sets g.gm1_hgw from the tables of the problem's order (call after g.gm1 and the tables
@@ -211,6 +221,14 @@ cudaError_t launch_sweep_r9(int dim, int dir, const GridInfo& g, const SweepArgs
 
 cudaError_t launch_combine(int dim, const GridInfo& g, const CombineArgs& a, cudaStream_t s);
 cudaError_t launch_max_speed(int dim, const GridInfo& g, const SpeedArgs& a, cudaStream_t s);
+// Single 2D problems below this many cells keep to FP64: a step is bound by its chain of launches
+// there, and looking for a front costs what the fixed-point sweep gains.
+constexpr long long kFrontCells = 128 * 128;
+inline bool looks_for_front(int dim, const GridInfo& g) {
+  return dim == 2 && (long long)g.nx * g.ny >= kFrontCells;
+}
+// front[0] of the status word from the strengths a 2D stage consumes.
+cudaError_t launch_strength(const GridInfo& g, const double* sx, const double* sy, DevState* st, cudaStream_t s);
 // All repair passes and the freeze of one stage in one cooperative launch (returns at once
 // when the stage update was physical everywhere; a grid barrier between passes).
 cudaError_t launch_repair_all(int dim, const GridInfo& g, const RepairArgs& a, cudaStream_t s);

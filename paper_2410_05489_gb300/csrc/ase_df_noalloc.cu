@@ -140,6 +140,9 @@ extern "C" ase_df_status ase_df_residual_noalloc(const ase_df_params* pin, const
 
   e = launch_state_kernel(st, 0, 0.0, s);  // clear the status word of the previous call
   if (e != cudaSuccess) return nfail(ASE_DF_E_CUDA, "status reset: %s", cudaGetErrorString(e));
+  const bool front = looks_for_front(p.ndim, g);
+  if (front && (e = launch_strength(g, sx_in, sy_in, st, s)) != cudaSuccess)
+    return nfail(ASE_DF_E_CUDA, "strength reduction: %s", cudaGetErrorString(e));
   for (int dir = 0; dir < p.ndim; ++dir) {
     SweepArgs a;
     a.W = W;
@@ -148,6 +151,7 @@ extern "C" ase_df_status ase_df_residual_noalloc(const ase_df_params* pin, const
     a.F = (dir == 0) ? Fx : Fy;
     a.s_out = (dir == 0) ? sx_out : sy_out;
     a.st = st;
+    if (front) a.front = &st->front[0];
     switch (p.order) {
       case 3: e = launch_sweep_r3(p.ndim, dir, g, a, *tab, s); break;
       case 5: e = launch_sweep_r5(p.ndim, dir, g, a, *tab, s); break;

@@ -11,6 +11,8 @@
 //            (r-1)/2 Gauss points (Sec. 2.1, Remark 2 of Sec. 3.1), the local
 //            Lax-Friedrichs flux and the discontinuity strength per Gauss point
 //            (Sec. 2.3, Sec. 3.1), the Gauss-weighted face flux and the face sigma.
+// In flows with a front the linear reconstructions of both phases run in fixed point on the
+// integer units (ase_df_fixed.cuh, sweep_tile).
 // The face fluxes go to global memory; the flux difference and the RK combination are
 // done by the combine kernel.
 //
@@ -51,7 +53,7 @@ template <int R, int DIM, int DIR, int TT, bool PLAN, int TN = (DIM == 2) ? 8 : 
 cudaError_t launch_grid(const GridInfo& g, const SweepArgs& a, const Tables& t, cudaStream_t s, dim3 grid,
                         const TilePlan& p) {
   using TL = Tile<R, DIM, TT, TN, NT>;
-  const size_t smem = TL::smem_doubles * sizeof(double);
+  const size_t smem = TL::sweep_doubles * sizeof(double);
   auto kern = sweep_kernel<R, DIM, DIR, TT, PLAN, TN, NT>;
   static std::atomic<unsigned long long> attr_done{0ull};
   cudaError_t e = ensure_smem_limit(kern, smem, attr_done);

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "ase_df_device.cuh"
+#include "ase_df_fixed.cuh"
 #include "ase_df_internal.cuh"
 
 namespace asedf {
@@ -23,19 +24,20 @@ struct Branch {
 };
 
 template <int R>
+__device__ __forceinline__ Branch linear_branch() {
+  return Branch{R, {1.0, 1.0, 1.0}, 1.0};
+}
+
+template <int R>
 __device__ __forceinline__ Branch select_branch(const double* s, double thres) {
   constexpr int K = (R - 1) / 2;
-  Branch b;
-  b.m = R;
-  b.a3[0] = b.a3[1] = b.a3[2] = 1.0;
-  b.a5 = 1.0;
+  Branch b = linear_branch<R>();
   // Smooth data without FP64 arithmetic: if every one of the 2K <= 8 strengths is at most
   // thres/16 (compared as unsigned bit patterns, so negative values and NaN fail), each
   // stencil sum is at most 8 thres/16 = thres/2 also after rounding (rounded addition is
   // monotone in its operands), so every sum is below thres and the branch is linear order R.
   {
-    const long long tb = dbits(thres);
-    const unsigned long long lim = ((tb >> 52) > 4) ? (unsigned long long)(tb - (4LL << 52)) : 0ull;
+    const unsigned long long lim = smooth_limit(thres);
     unsigned long long mx = (unsigned long long)dbits(s[0]);
 #pragma unroll
     for (int t = 1; t < 2 * K; ++t) mx = max(mx, (unsigned long long)dbits(s[t]));
@@ -228,6 +230,9 @@ struct Tile {
   static constexpr size_t queue_offset =
       (size_t)C * NB * NA + 2 * (size_t)C * NB * NQ + (size_t)NB * NSN + (DIM == 2 ? (size_t)NQ * NST : 0);
   static constexpr size_t smem_doubles = queue_offset + ((size_t)QCAP + 2 + 1) / 2;
+  // 2D sweeps, after the queue: a flag (2 ints) and 8 ints per warp (TileSpan)
+  static constexpr size_t span_offset = smem_doubles;
+  static constexpr size_t sweep_doubles = smem_doubles + (DIM == 2 ? 1 + (size_t)(NT / 32) * 4 : 0);
 };
 
 // Quotient and remainder by a tile's run-time line count n (at most 127) of an index below 2^13, by
@@ -264,9 +269,119 @@ __device__ __forceinline__ bool defer_item(bool defer, int item, int* queue, uns
   return defer;
 }
 
+// One component of one staged line in fixed point at the tile's exponent e: the order-R linear
+// reconstruction of its NQ cells at both faces (the two end cells at one).  The line's cell
+// averages are converted once and serve all of its stencils.
+template <int R, int NA, int NQ>
+__device__ __forceinline__ void fix_line(const double* v, int e, Limbs* qp, Limbs* qm) {
+  constexpr int K = (R - 1) / 2;
+  const FixWeights& F = kFixW[(R - 3) / 2];
+  Limbs m[NA];
+#pragma unroll
+  for (int t = 0; t < NA; ++t) m[t] = fix_from_double(v[t], e);
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    if (q < NQ - 1) {
+      FixSum s = fix_zero();
+#pragma unroll
+      for (int t = 0; t <= 2 * K; ++t) fix_mad(s, m[q + t], F.fh[t], F.fl[t]);
+      qp[q] = fix_split(fix_value(s));
+    }
+    if (q > 0) {
+      FixSum s = fix_zero();
+#pragma unroll
+      for (int t = 0; t <= 2 * K; ++t) fix_mad(s, m[q + t], F.fh[2 * K - t], F.fl[2 * K - t]);
+      qm[q] = fix_split(fix_value(s));
+    }
+  }
+}
+
+// Gauss-point values of the order-R linear branch from the normal values Q (stride NQ) of lines
+// -K .. K: the even and odd sums of lin_gauss_sym in fixed point.  The limbs add without carry.
+template <int R, int G, int NQ>
+__device__ __forceinline__ void fix_gauss(const Limbs* Q, int e, double* out) {
+  constexpr int K = (R - 1) / 2;
+  const FixWeights& F = kFixW[(R - 3) / 2];
+  Limbs S[K + 1], D[K + 1];
+  S[0] = Q[0];
+#pragma unroll
+  for (int t = 1; t <= K; ++t) {
+    const Limbs a = Q[t * NQ], b = Q[-t * NQ];
+    S[t] = Limbs{a.h + b.h, a.l + b.l};
+    D[t] = Limbs{a.h - b.h, a.l - b.l};
+  }
+#pragma unroll
+  for (int g = 0; g < (G + 1) / 2; ++g) {
+    FixSum E = fix_zero();
+#pragma unroll
+    for (int t = 0; t <= K; ++t) fix_mad(E, S[t], F.eh[g][t], F.el[g][t]);
+    const long long ev = fix_value(E);
+    if (2 * g + 1 == G) {
+      out[g] = fix_to_double(ev, e);  // middle point
+    } else {
+      FixSum O = fix_zero();
+#pragma unroll
+      for (int t = 1; t <= K; ++t) fix_mad(O, D[t], F.oh[g][t], F.ol[g][t]);
+      const long long ov = fix_value(O);
+      out[g] = fix_to_double(ev + ov, e);
+      out[G - 1 - g] = fix_to_double(ev - ov, e);
+    }
+  }
+}
+
+// What a tile's staged cell averages span, on the high words of the doubles: largest and smallest
+// of density and energy, largest momentum magnitude (each thread its own, then the CTA's).
+struct TileSpan {
+  int rmax = 0, rmin = 0x7fffffff, emax = 0, emin = 0x7fffffff, mmax = 0;
+  __device__ __forceinline__ void add(int c, int last, double v) {
+    const int hi = (int)(dbits(v) >> 32);
+    if (c == 0) { rmax = max(rmax, hi & 0x7fffffff); rmin = min(rmin, hi); }
+    else if (c == last) { emax = max(emax, hi & 0x7fffffff); emin = min(emin, hi); }
+    else mmax = max(mmax, hi & 0x7fffffff);
+  }
+  // s_part: 8 ints per warp; store before and load after a barrier
+  __device__ __forceinline__ void store(int* s_part) const {
+    const int v[5] = {__reduce_max_sync(0xffffffffu, rmax), __reduce_min_sync(0xffffffffu, rmin),
+                      __reduce_max_sync(0xffffffffu, emax), __reduce_min_sync(0xffffffffu, emin),
+                      __reduce_max_sync(0xffffffffu, mmax)};
+    if ((threadIdx.x & 31) == 0)
+      for (int k = 0; k < 5; ++k) s_part[(threadIdx.x >> 5) * 8 + k] = v[k];
+  }
+  __device__ __forceinline__ void load(const int* s_part, int warps) {
+    for (int w = 0; w < warps; ++w) {
+      rmax = max(rmax, s_part[w * 8]);
+      rmin = min(rmin, s_part[w * 8 + 1]);
+      emax = max(emax, s_part[w * 8 + 2]);
+      emin = min(emin, s_part[w * 8 + 3]);
+      mmax = max(mmax, s_part[w * 8 + 4]);
+    }
+  }
+  // density and energy positive and within kFixRange binades each, nothing huge or non-finite
+  __device__ __forceinline__ bool fits() const {
+    return rmin > 0 && emin > 0 && exp_of(rmax) - exp_of(rmin) <= kFixRange &&
+           exp_of(emax) - exp_of(emin) <= kFixRange &&
+           max(exp_of(rmax), max(exp_of(emax), exp_of(mmax))) <= kFixMaxExp;
+  }
+};
+
 // One tile: faces a0 .. a0+TN-1 along the sweep on lines b0 .. b0+tt-1, 1 <= tt <= TT
-// (threadIdx.x is the worker index); smem holds Tile<R, DIM, TT>::smem_doubles doubles,
+// (threadIdx.x is the worker index); smem holds Tile<R, DIM, TT>::sweep_doubles doubles,
 // laid out for TT lines whatever tt is.
+//
+// 2D flows with a front (some face strength of the problem is beyond smooth_limit, below which
+// every branch is linear) take both reconstructions in fixed point on the integer units
+// (ase_df_fixed.cuh) in the tiles whose density and energy span few binades (TileSpan::fits),
+// wherever the branch is the linear one of order R; the FP64 pipe is left to the Gauss points.
+// The other branches run in FP64 in second passes over queues of such cells and faces.  Normal
+// values are then kept in shared memory as limbs at the tile's exponents.  An order-9 face then
+// takes 287 FP64 instructions instead of 586 (pipe 72 % busy, the rest waits on the 16 resident
+// warps).  Measured, FP64 -> fixed point: Configuration 3 512^2 order 5, one step, 1350 -> 1013 us;
+// the 1600 x 800 order-9 jet residual 3700 -> 2653 us; 64 mixed problems 14.5 -> 11.1 ms.  Exponents
+// per line with aligned sums measured 1046 / 2708 us / 13.0 ms: the alignment costs instructions,
+// and lines crossing a strong front made their tiles slower than plain FP64.
+// Flows without a front stay in FP64 to the bit: their strengths are differences of two
+// reconstructions that agree to rounding (1e-12 made of 1e-16 parts on a fine smooth grid), so
+// any other rounding of a state, however exact, shows in the fifth digit of the strengths.
 template <int R, int DIM, int DIR, int TT_ = (DIM == 2) ? 64 : 1, int TN_ = (DIM == 2) ? 8 : 255, int NT_ = 256>
 __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& args, const Tables& T, int a0,
                                            int b0, int tt, double* smem) {
@@ -296,6 +411,14 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   int* s_queue = reinterpret_cast<int*>(smem + TL::queue_offset);
   unsigned int* s_qn = reinterpret_cast<unsigned int*>(s_queue + TL::QCAP);
   if (tid < 2) s_qn[tid] = 0u;
+  // fixed point: a flag for a value that does not fit, and the warps' spans
+  int* s_any = reinterpret_cast<int*>(smem + TL::span_offset);
+  int* s_part = s_any + 2;
+  if (DIM == 2 && tid == 0) *s_any = 0;
+  Limbs* iQP = reinterpret_cast<Limbs*>(sQP);
+  Limbs* iQM = reinterpret_cast<Limbs*>(sQM);
+  const bool front = DIM == 2 && args.front != nullptr && *args.front != 0u;
+  const unsigned long long limit = smooth_limit(g.thres);
   // ---- staging: consecutive threads take consecutive addresses along the direction in which the
   // arrays are contiguous (the sweep for x-faces, the lines for y-faces) ----
   static_assert(NA * NB < (1 << 13) && NB < 128, "LineDiv range");
@@ -304,6 +427,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   // a tile whose halo lies inside the grid needs none of the boundary's index maps
   const bool inside = DIM == 2 && a0 - 1 - K >= 0 && a0 + TN - 1 + K < n && b0 - KT >= 0 && b0 + tt + KT <= mlin;
   // cell averages: cells a0-1-K .. a0+TN-1+K, lines b0-KT .. b0+tt+KT-1
+  TileSpan span;
   for (int idx = tid; idx < nb * NA; idx += NT) {
     int bb, aa;
     if (DIR == 0) { aa = idx % NA; bb = idx / NA; }
@@ -313,13 +437,36 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
     if (inside) {
       const double* src = args.W + (size_t)b * stb + (size_t)a * sta;
 #pragma unroll
-      for (int c = 0; c < C; ++c) dst[c * NB * NA] = __ldg(src + (size_t)c * g.nx * g.ny);
+      for (int c = 0; c < C; ++c) {
+        const double v = __ldg(src + (size_t)c * g.nx * g.ny);
+        dst[c * NB * NA] = v;
+        if (DIM == 2) span.add(c, C - 1, v);
+      }
     } else {
       const int i = (DIR == 0) ? a : b, j = (DIR == 0) ? b : a;
 #pragma unroll 1
-      for (int c = 0; c < C; ++c) dst[c * NB * NA] = fetch_w(g, args.W, c, i, j, ts);
+      for (int c = 0; c < C; ++c) {
+        const double v = fetch_w(g, args.W, c, i, j, ts);
+        dst[c * NB * NA] = v;
+        if (DIM == 2) span.add(c, C - 1, v);
+      }
     }
   }
+  if (front) {
+    if constexpr (DIM == 2 && TT == 32) {
+      // a tile of 32 lines takes the exponents of the 64-line tile it is half of, so that the tile
+      // shape does not change the results: the other half's lines are looked at, not staged
+      const int bx = (b0 & 32) ? b0 - 32 - KT : b0 + 32 + KT;
+      for (int idx = tid; idx < 32 * NA; idx += NT) {
+        const int a = a0 - 1 - K + ((DIR == 0) ? idx % NA : idx / 32), b = bx + ((DIR == 0) ? idx / NA : idx % 32);
+#pragma unroll 1
+        for (int c = 0; c < C; ++c)
+          span.add(c, C - 1, (DIR == 0) ? fetch_w(g, args.W, c, a, b, ts) : fetch_w(g, args.W, c, b, a, ts));
+      }
+    }
+    span.store(s_part);
+  }
+  bool rough = false;  // a strength beyond the limit below which every branch is linear of order R
   // normal face strengths: faces a0-K .. a0+TN-1+K of every staged line
   for (int idx = tid; idx < nb * NSN; idx += NT) {
     int fa, bb;
@@ -330,6 +477,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
     if (inside) v = __ldg(args.s_norm + ((DIR == 0) ? (size_t)b * (g.nx + 1) + f : (size_t)f * g.nx + b));
     else v = (DIR == 0) ? sigma_x_at(g, args.s_norm, f, b) : sigma_y_at(g, args.s_norm, f, b);
     sSn[bb * NSN + fa] = v;
+    rough |= is_front(v, limit);
   }
   // tangential face strengths of the reconstructing cells' columns: faces b0-K+1 .. b0+tt+K-1
   if (DIM == 2) {
@@ -344,58 +492,113 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       if (inside) v = __ldg(args.s_tan + ((DIR == 0) ? (size_t)f * g.nx + a : (size_t)a * (g.nx + 1) + f));
       else v = (DIR == 0) ? sigma_y_at(g, args.s_tan, f, a) : sigma_x_at(g, args.s_tan, f, a);
       sSt[qa * NST + fb] = v;
+      rough |= is_front(v, limit);
     }
   }
-  __syncthreads();
+  rough = __syncthreads_or(rough);
+  // a tile without such a strength needs no branch choice
+  auto branch = [&](const double* s) { return rough ? select_branch<R>(s, g.thres) : linear_branch<R>(); };
 
   // ---- phase 1: normal reconstruction of cells a0-1 .. a0+TN-1 on all staged lines ----
-  // Interior cells (qa = 1 .. NQ-2) serve a face on each side and are evaluated at both
-  // xi = 0 and xi = -1; the two end cells serve one tile face each (qa = 0: its xi = 0
-  // value, the left state of face a0; qa = NQ-1: its xi = -1 value), so they come last in
-  // the work list and evaluate one point.
-  // Fallback items are deferred (defer_item) and done in a second pass.
+  // Interior cells serve a face on each side and are evaluated at both xi = 0 and xi = -1; the
+  // two end cells serve one tile face each (qa = 0: its xi = 0 value, the left state of face
+  // a0; qa = NQ-1: its xi = -1 value).
+  bool fixed = false;
+  int ex[3];  // exponents of density, momentum, energy
+  if (front) {
+    span.load(s_part, NT / 32);
+    fixed = span.fits();
+    ex[0] = fix_exponent(exp_of(span.rmax));
+    ex[1] = fix_exponent(exp_of(span.mmax));
+    ex[2] = fix_exponent(exp_of(span.emax));
+  }
+  auto comp_exp = [&](int c) { return c == 0 ? ex[0] : c == C - 1 ? ex[2] : ex[1]; };
+  if (fixed) {
+    for (int it = tid; it < C * nb; it += NT) {
+      int c, bb;
+      dnb.split(it, c, bb);
+      const int row = c * NB + bb;
+      fix_line<R, NA, NQ>(sW + row * NA, comp_exp(c), iQP + row * NQ, iQM + row * NQ);
+    }
+    if (rough)
+      for (int it = tid; it < NQ * nb; it += NT)
+        defer_item(select_branch<R>(sSn + (it / NQ) * NSN + it % NQ, g.thres).m != R, it, s_queue, &s_qn[0]);
+    __syncthreads();
+    // cells of another branch, in FP64, then converted
+    const int nq = (int)s_qn[0];
+    if (nq > 0) {
+      for (int k = tid; k < nq; k += NT) {
+        const int it = s_queue[k];
+        const int bb = it / NQ, qa = it % NQ;
+        const Branch br = select_branch<R>(sSn + bb * NSN + qa, g.thres);
 #pragma unroll 1
-  for (int pass = 0; pass < 2; ++pass) {
-    const int count = (pass == 0) ? NQ * nb : (int)s_qn[0];
-    for (int k = tid; k < count; k += NT) {
-      const int it = (pass == 0) ? k : s_queue[k];
-      int qa, bb, pt;  // pt -1: an interior cell, both points; 0 / 1: an end cell, one point
-      if (it < (NQ - 2) * nb) {
-        if (DIR == 0) { qa = 1 + it % (NQ - 2); bb = it / (NQ - 2); }
-        else { dnb.split(it, qa, bb); ++qa; }
-        pt = -1;
-      } else {
-        dnb.split(it - (NQ - 2) * nb, pt, bb);  // pt 0: cell qa = 0 at xi = 0; 1: qa = NQ-1 at xi = -1
-        qa = pt * (NQ - 1);
-      }
-      const Branch br = select_branch<R>(sSn + bb * NSN + qa, g.thres);
-      if (R >= 5 && pass == 0 && defer_item(br.m == 0, it, s_queue, &s_qn[0])) continue;
-      if (pt < 0) {
-#pragma unroll
         for (int c = 0; c < C; ++c) {
-          const double* v = sW + (c * NB + bb) * NA + qa + K;  // W_0 of this cell
+          const int row = c * NB + bb, e = comp_exp(c);
           double out[2];
-          recon_eval<R, 2>(v, 1, br, T, 0, out);
-          sQP[(c * NB + bb) * NQ + qa] = out[0];
-          sQM[(c * NB + bb) * NQ + qa] = out[1];
-        }
-      } else {
-        double* dst = pt ? sQM : sQP;
+          recon_eval<R, 2>(sW + row * NA + qa + K, 1, br, T, 0, out);
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-          const double* v = sW + (c * NB + bb) * NA + qa + K;
-          double out[1];
-          recon_eval<R, 1>(v, 1, br, T, pt, out);
-          dst[(c * NB + bb) * NQ + qa] = out[0];
+          for (int q = 0; q < 2; ++q) {
+            if (exp_of((int)(dbits(out[q]) >> 32) & 0x7fffffff) > e + 1) *s_any = 1;  // e.g. non-finite
+            else (q == 0 ? iQP : iQM)[row * NQ + qa] = fix_split(fix_join(fix_from_double(out[q], e)));
+          }
         }
+      }
+      __syncthreads();
+      if (*s_any) {  // the whole tile in FP64
+        fixed = false;
+        __syncthreads();
+        if (tid == 0) s_qn[0] = 0u;
+        __syncthreads();
       }
     }
-    __syncthreads();  // pass 0: the queue is complete; last pass: phase 1 is done
-    if (R < 5 || s_qn[0] == 0u) break;
+  }
+  if (!fixed) {
+    // FP64: the end cells come last in the work list and evaluate one point; fallback cells are
+    // deferred (defer_item) and done in a second pass
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+      const int count = (pass == 0) ? NQ * nb : (int)s_qn[0];
+      for (int k = tid; k < count; k += NT) {
+        const int it = (pass == 0) ? k : s_queue[k];
+        int qa, bb, pt;  // pt -1: an interior cell, both points; 0 / 1: an end cell, one point
+        if (it < (NQ - 2) * nb) {
+          if (DIR == 0) { qa = 1 + it % (NQ - 2); bb = it / (NQ - 2); }
+          else { dnb.split(it, qa, bb); ++qa; }
+          pt = -1;
+        } else {
+          dnb.split(it - (NQ - 2) * nb, pt, bb);  // pt 0: cell qa = 0 at xi = 0; 1: qa = NQ-1 at xi = -1
+          qa = pt * (NQ - 1);
+        }
+        const Branch br = branch(sSn + bb * NSN + qa);
+        if (R >= 5 && rough && pass == 0 && defer_item(br.m == 0, it, s_queue, &s_qn[0])) continue;
+        if (pt < 0) {
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            const double* v = sW + (c * NB + bb) * NA + qa + K;  // W_0 of this cell
+            double out[2];
+            recon_eval<R, 2>(v, 1, br, T, 0, out);
+            sQP[(c * NB + bb) * NQ + qa] = out[0];
+            sQM[(c * NB + bb) * NQ + qa] = out[1];
+          }
+        } else {
+          double* dst = pt ? sQM : sQP;
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            const double* v = sW + (c * NB + bb) * NA + qa + K;
+            double out[1];
+            recon_eval<R, 1>(v, 1, br, T, pt, out);
+            dst[(c * NB + bb) * NQ + qa] = out[0];
+          }
+        }
+      }
+      __syncthreads();  // pass 0: the queue is complete; last pass: phase 1 is done
+      if (R < 5 || s_qn[0] == 0u) break;
+    }
   }
 
   // ---- phase 2: faces ----
-  // Faces with a fallback tangential reconstruction on either side are deferred (2D).
+  // 2D: faces with a fallback tangential reconstruction on either side (fixed point: with any but
+  // the order-R linear one) are deferred.
   const LineDiv dtt(tt);
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
@@ -409,32 +612,64 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       if (f > n || b >= mlin) continue;
       Branch bt[2];
       if (DIM == 2) {
-        bt[0] = select_branch<R>(sSt + fa * NST + tb, g.thres);  // the columns of the two states
-        bt[1] = select_branch<R>(sSt + (fa + 1) * NST + tb, g.thres);
-        if (R >= 5 && pass == 0 && defer_item(bt[0].m == 0 || bt[1].m == 0, it, s_queue, &s_qn[1])) continue;
+        bt[0] = branch(sSt + fa * NST + tb);  // the columns of the two states
+        bt[1] = branch(sSt + (fa + 1) * NST + tb);
+        if (rough && pass == 0) {
+          const bool defer = fixed ? bt[0].m != R || bt[1].m != R : R >= 5 && (bt[0].m == 0 || bt[1].m == 0);
+          if (defer_item(defer, it, s_queue, &s_qn[1])) continue;
+        }
       }
       double st[2][G][C];
+      if (counting) {
 #pragma unroll
-      for (int side = 0; side < 2; ++side) {
-        const int qa = fa + side;  // left state: cell f-1 (plus face); right: cell f (minus face)
-        const double* Q = side == 0 ? sQP : sQM;
-        if (counting) {  // the normal branch of this state's cell, as phase 1 chose it
-          const Branch bn = select_branch<R>(sSn + (tb + KT) * NSN + qa, g.thres);
+        for (int side = 0; side < 2; ++side) {  // the normal branch as phase 1 chose it, the tangential one
+          const Branch bn = select_branch<R>(sSn + (tb + KT) * NSN + fa + side, g.thres);
           atomicAdd(&hist_s[branch_slot(bn.m)], 1u);
+          if (DIM == 2) atomicAdd(&hist_s[branch_slot(bt[side].m)], 1u);
         }
-        if (DIM == 2) {
-          if (counting) atomicAdd(&hist_s[branch_slot(bt[side].m)], 1u);
+      }
+      // left state: cell f-1 (plus face); right: cell f (minus face)
+      if constexpr (DIM == 2) {
+        if (!fixed) {
+#pragma unroll
+          for (int side = 0; side < 2; ++side)
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+              double out[G];
+              tang_eval<R, G>((side == 0 ? sQP : sQM) + (c * NB + tb + K) * NQ + fa + side, NQ, bt[side], T, out);
+#pragma unroll
+              for (int q = 0; q < G; ++q) st[side][q][c] = out[q];
+            }
+        } else if (pass == 0) {
 #pragma unroll
           for (int c = 0; c < C; ++c) {
-            const double* v = Q + (c * NB + tb + K) * NQ + qa;
-            double out[G];
-            tang_eval<R, G>(v, NQ, bt[side], T, out);
 #pragma unroll
-            for (int q = 0; q < G; ++q) st[side][q][c] = out[q];
+            for (int side = 0; side < 2; ++side) {
+              double out[G];
+              fix_gauss<R, G, NQ>((side == 0 ? iQP : iQM) + (c * NB + tb + K) * NQ + fa + side, comp_exp(c), out);
+#pragma unroll
+              for (int q = 0; q < G; ++q) st[side][q][c] = out[q];
+            }
           }
         } else {
 #pragma unroll
-          for (int c = 0; c < C; ++c) st[side][0][c] = Q[c * NQ + qa];
+          for (int c = 0; c < C; ++c)
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+              double v[2 * K + 1], out[G];
+#pragma unroll
+              for (int t = 0; t <= 2 * K; ++t)
+                v[t] = fix_to_double(fix_join((side == 0 ? iQP : iQM)[(c * NB + tb + t) * NQ + fa + side]), comp_exp(c));
+              tang_eval<R, G>(v + K, 1, bt[side], T, out);
+#pragma unroll
+              for (int q = 0; q < G; ++q) st[side][q][c] = out[q];
+            }
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          st[0][0][c] = sQP[c * NQ + fa];
+          st[1][0][c] = sQM[c * NQ + fa + 1];
         }
       }
       // cell averages either side of the face (read by a Gauss point only if it falls back)
@@ -457,6 +692,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         if (counting) atomicAdd(&hist_s[kBranchSlots - 1], nfb);
       }
       const double sface = (G == 1) ? ssum : ssum * (1.0 / G);
+      if (DIM == 2 && args.front_out != nullptr && is_front(sface, limit)) *args.front_out = 1u;
       if (DIR == 0) {
 #pragma unroll
         for (int c = 0; c < C; ++c) args.F[((size_t)c * g.ny + b) * (g.nx + 1) + f] = Fs[c];
@@ -467,7 +703,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         args.s_out[(size_t)f * g.nx + b] = sface;
       }
     }
-    if (DIM == 1 || R < 5 || pass == 1) break;
+    if (DIM == 1 || pass == 1) break;
     __syncthreads();  // the queue is complete
     if (s_qn[1] == 0u) break;
   }
