@@ -527,12 +527,13 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
     // cells of another branch, in FP64, then converted
     const int nq = (int)s_qn[0];
     if (nq > 0) {
-      for (int k = tid; k < nq; k += NT) {
-        const int it = s_queue[k];
+      const int cs = nq * C <= NT ? C : 1;  // threads per cell (as below)
+      for (int k = tid; k < nq * cs; k += NT) {
+        const int it = s_queue[k / cs];
         const int bb = it / NQ, qa = it % NQ;
         const Branch br = select_branch<R>(sSn + bb * NSN + qa, g.thres);
 #pragma unroll 1
-        for (int c = 0; c < C; ++c) {
+        for (int c = k % cs; c < C; c += cs) {
           const int row = c * NB + bb, e = comp_exp(c);
           double out[2];
           recon_eval<R, 2>(sW + row * NA + qa + K, 1, br, T, 0, out);
@@ -592,7 +593,30 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         }
       }
       __syncthreads();  // pass 0: the queue is complete; last pass: phase 1 is done
-      if (R < 5 || s_qn[0] == 0u) break;
+      if (R < 5 || s_qn[0] == 0u || pass == 1) break;
+      const int nq = (int)s_qn[0];
+      if (nq * C > NT) continue;
+      // a short queue: one component of a cell per thread.  The fallback of one component is some
+      // 200 dependent FP64 instructions, and the tile waits for its slowest thread (Sod tube of 200
+      // cells, first sweep 42.7 -> 19.6 us, later ones 11.7 -> 10.6); a long queue keeps one thread per cell, which chooses
+      // the branch (and divides for its DF factors) once.
+      for (int k = tid; k < nq * C; k += NT) {
+        const int it = s_queue[k / C], c = k % C;
+        int bb, qa;
+        if (it < (NQ - 2) * nb) {
+          if (DIR == 0) { qa = 1 + it % (NQ - 2); bb = it / (NQ - 2); }
+          else { dnb.split(it, qa, bb); ++qa; }
+        } else {
+          dnb.split(it - (NQ - 2) * nb, qa, bb);
+          qa *= NQ - 1;
+        }
+        double out[2];  // an end cell's value at its outer face is formed too and not read
+        recon_eval<R, 2>(sW + (c * NB + bb) * NA + qa + K, 1, select_branch<R>(sSn + bb * NSN + qa, g.thres), T, 0, out);
+        sQP[(c * NB + bb) * NQ + qa] = out[0];
+        sQM[(c * NB + bb) * NQ + qa] = out[1];
+      }
+      __syncthreads();
+      break;
     }
   }
 
