@@ -6,6 +6,7 @@
 
 #include <cuda_runtime.h>
 
+#include "ase_df_imul.cuh"
 #include "ase_df_internal.cuh"
 
 namespace asedf {
@@ -71,6 +72,7 @@ __device__ __forceinline__ double rcp_pos(double x) {
 // approximation of x scaled by an even power of two into [1, 4).  Then one third-order
 // step: with r = 1 - x y0^2, 1/sqrt(x) = y0 (1 - r)^(-1/2) = y0 (1 + r/2 + 3 r^2 / 8 + ...),
 // so y1 = y0 + y0 r (1/2 + 3 r / 8), error O(r^3) < 2^-62 before rounding.
+template <bool INT = false>
 __device__ __forceinline__ double rsqrt_pos(double x) {
   const long long b = dbits(x);
   const int ex = (int)((b >> 52) & 0x7ff);
@@ -85,9 +87,9 @@ __device__ __forceinline__ double rsqrt_pos(double x) {
   const unsigned sb = __float_as_uint(sf);
   const long long es = (long long)((sb >> 23) & 0xffu) - 127 + 1023 - k;
   const double y0 = __longlong_as_double((es << 52) | ((long long)(sb & 0x7fffffu) << 29));
-  const double h = x * y0;
+  const double h = lf_mul<INT>(x, y0);
   const double r = fma(-h, y0, 1.0);
-  return fma(y0 * r, fma(r, 0.375, 0.5), y0);
+  return fma(lf_mulz<INT>(r, y0), fma(r, 0.375, 0.5), y0);
 }
 
 // cell index 0..n-1 of a (ghost) cell; a reflecting wall mirrors about its face (the
@@ -176,6 +178,8 @@ __device__ __forceinline__ double sigma_y_at(const GridInfo& g, const double* __
 //   - c^2 = gamma p / rho = gg1 p' / rho and 1/c from a seeded reciprocal square root;
 //     c = c^2 / c;
 //   - 1/p' = gg1 (1/rho) (1/c)^2 gives the pressure term of sigma without a reciprocal;
+//   - the 25 products that are no part of a multiply-add (28 instructions) can be formed on the
+//     integer units (INT; ase_df_imul.cuh), bit for bit the same;
 //   - the flux sum F_l + F_r - lambda (q_r - q_l) is formed per component as
 //     q_l (u_l + lambda) + q_r (u_r - lambda) + pressure terms, and accumulated into the
 //     caller's Gauss sum in the same FMAs.
@@ -188,19 +192,19 @@ struct LfPrims {
   double irL, irR, unL, unR, utL, utR, pL, pR;
 };
 
-template <int C, int NI, int TI>
+template <int C, int NI, int TI, bool INT = false>
 __device__ __forceinline__ LfPrims lf_primitives(const double* a, const double* b) {
   LfPrims s;
-  const double irr = rcp_pos(a[0] * b[0]);
-  s.irL = b[0] * irr;
-  s.irR = a[0] * irr;
-  s.unL = a[NI] * s.irL;
-  s.unR = b[NI] * s.irR;
-  double kL = a[NI] * s.unL, kR = b[NI] * s.unR;  // |m|^2 / rho
+  const double irr = rcp_pos(lf_mul<INT>(a[0], b[0]));
+  s.irL = lf_mul<INT>(b[0], irr);
+  s.irR = lf_mul<INT>(a[0], irr);
+  s.unL = lf_mulz<INT>(a[NI], s.irL);
+  s.unR = lf_mulz<INT>(b[NI], s.irR);
+  double kL = lf_mulz<INT>(a[NI], s.unL), kR = lf_mulz<INT>(b[NI], s.unR);  // |m|^2 / rho
   s.utL = s.utR = 0.0;
   if (C == 4) {
-    s.utL = a[TI] * s.irL;
-    s.utR = b[TI] * s.irR;
+    s.utL = lf_mulz<INT>(a[TI], s.irL);
+    s.utR = lf_mulz<INT>(b[TI], s.irR);
     kL = fma(a[TI], s.utL, kL);
     kR = fma(b[TI], s.utR, kR);
   }
@@ -214,10 +218,56 @@ __device__ __forceinline__ bool lf_physical(double rhoL, double rhoR, const LfPr
   return pos_finite(rhoL) && pos_finite(rhoR) && pos_finite(s.pL) && pos_finite(s.pR);
 }
 
-template <int C, int NI, int TI>
+// Flux and strength of a point from its states and their primitives.
+template <int C, int NI, int TI, bool INT = false>
+__device__ __forceinline__ void lf_flux(const double* a, const double* b, const LfPrims& s, bool ok, double gg1,
+                                        double w, double gw, double* Fs, double& sigma) {
+  const double irL = s.irL, irR = s.irR, unL = s.unL, unR = s.unR, utL = s.utL, utR = s.utR;
+  const double pL = s.pL, pR = s.pR;
+  const double c2L = lf_mul<INT>(lf_mul<INT>(gg1, pL), irL), c2R = lf_mul<INT>(lf_mul<INT>(gg1, pR), irR);
+  const double icL = rsqrt_pos<INT>(c2L), icR = rsqrt_pos<INT>(c2R);
+  // lambda = max(|u_n| + c) with c = c^2 / c
+  const double lam = max_nonneg(fma(c2L, icL, fabs(unL)), fma(c2R, icR, fabs(unR)));
+  const double alL = lf_mulz<INT>(unL + lam, w), alR = lf_mulz<INT>(unR - lam, w);
+  Fs[0] = fma(a[0], alL, fma(b[0], alR, Fs[0]));
+  Fs[NI] = fma(a[NI], alL, fma(b[NI], alR, fma(gw, pL + pR, Fs[NI])));
+  if (C == 4) Fs[TI] = fma(a[TI], alL, fma(b[TI], alR, Fs[TI]));
+  Fs[C - 1] = fma(a[C - 1], alL, fma(b[C - 1], alR, fma(gw, fma(unL, pL, lf_mulz<INT>(unR, pR)), Fs[C - 1])));
+  if (ok) {
+    // sigma = |dp| (1/p_l + 1/p_r) + (dMa_n)^2 + (dMa_t)^2, Ma = u / c
+    const double dmn = fma(unL, icL, -lf_mulz<INT>(unR, icR));
+    double s = lf_mulz<INT>(dmn, dmn);
+    if (C == 4) {
+      const double dmt = fma(utL, icL, -lf_mulz<INT>(utR, icR));
+      s = fma(dmt, dmt, s);
+    }
+    const double tL = lf_mul<INT>(irL, icL), tR = lf_mul<INT>(irR, icR);
+    const double ip = fma(tL, icL, lf_mul<INT>(tR, icR));  // (1/p'_l + 1/p'_r) / gg1
+    sigma = fma(lf_mulz<INT>(fabs(pL - pR), gg1), ip, s);
+  } else {
+    sigma = kSigmaBig;
+  }
+}
+
+// ints (with INT): the products on the integer units.  They are there for states within imul_pos /
+// imul_any, which bound every operand of a point; others, non-physical ones among them, take the
+// FP64 unit.
+template <int C, int NI, int TI, bool INT = false>
 __device__ __forceinline__ bool lf_point_acc(const double* qa, const double* qb, const double* ca,
                                              const double* cb, int cs, double gm1, double gg1, double w,
-                                             double gw, double* Fs, double& sigma) {
+                                             double gw, bool ints, double* Fs, double& sigma) {
+  if (INT) {
+    bool in = ints && imul_pos(qa[0]) && imul_pos(qb[0]) && imul_pos(gg1);
+#pragma unroll
+    for (int c = 1; c < C - 1; ++c) in = in && imul_any(qa[c]) && imul_any(qb[c]);
+    if (in) {
+      const LfPrims s = lf_primitives<C, NI, TI, true>(qa, qb);
+      if (imul_pos(s.pL) && imul_pos(s.pR)) {
+        lf_flux<C, NI, TI, true>(qa, qb, s, true, gg1, w, gw, Fs, sigma);
+        return false;
+      }
+    }
+  }
   double a[C], b[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) {
@@ -234,31 +284,7 @@ __device__ __forceinline__ bool lf_point_acc(const double* qa, const double* qb,
     }
     s = lf_primitives<C, NI, TI>(a, b);
   }
-  const double irL = s.irL, irR = s.irR, unL = s.unL, unR = s.unR, utL = s.utL, utR = s.utR;
-  const double pL = s.pL, pR = s.pR;
-  const double c2L = (gg1 * pL) * irL, c2R = (gg1 * pR) * irR;
-  const double icL = rsqrt_pos(c2L), icR = rsqrt_pos(c2R);
-  // lambda = max(|u_n| + c) with c = c^2 / c
-  const double lam = max_nonneg(fma(c2L, icL, fabs(unL)), fma(c2R, icR, fabs(unR)));
-  const double alL = w * (unL + lam), alR = w * (unR - lam);
-  Fs[0] = fma(a[0], alL, fma(b[0], alR, Fs[0]));
-  Fs[NI] = fma(a[NI], alL, fma(b[NI], alR, fma(gw, pL + pR, Fs[NI])));
-  if (C == 4) Fs[TI] = fma(a[TI], alL, fma(b[TI], alR, Fs[TI]));
-  Fs[C - 1] = fma(a[C - 1], alL, fma(b[C - 1], alR, fma(gw, fma(unL, pL, unR * pR), Fs[C - 1])));
-  if (ok) {
-    // sigma = |dp| (1/p_l + 1/p_r) + (dMa_n)^2 + (dMa_t)^2, Ma = u / c
-    const double dmn = fma(unL, icL, -unR * icR);
-    double s = dmn * dmn;
-    if (C == 4) {
-      const double dmt = fma(utL, icL, -utR * icR);
-      s = fma(dmt, dmt, s);
-    }
-    const double tL = irL * icL, tR = irR * icR;
-    const double ip = fma(tL, icL, tR * icR);  // (1/p'_l + 1/p'_r) / gg1
-    sigma = fma(gg1 * fabs(pL - pR), ip, s);
-  } else {
-    sigma = kSigmaBig;
-  }
+  lf_flux<C, NI, TI>(a, b, s, ok, gg1, w, gw, Fs, sigma);
   return !ok;
 }
 
@@ -270,7 +296,7 @@ __device__ __forceinline__ bool lf_point(const double* qa, const double* qb, con
                                          double& sigma) {
 #pragma unroll
   for (int c = 0; c < C; ++c) F2[c] = 0.0;
-  return lf_point_acc<C, NI, TI>(qa, qb, ca, cb, cs, gm1, gg1, 1.0, gm1, F2, sigma);
+  return lf_point_acc<C, NI, TI>(qa, qb, ca, cb, cs, gm1, gg1, 1.0, gm1, false, F2, sigma);
 }
 
 }  // namespace

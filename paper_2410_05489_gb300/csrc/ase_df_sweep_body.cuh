@@ -391,6 +391,17 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   constexpr int NA = TL::NA, NB = TL::NB, NQ = TL::NQ, NSN = TL::NSN, NST = TL::NST;
   constexpr int NI = (DIR == 0) ? 1 : 2;  // normal momentum component
   constexpr int TI = (DIR == 0) ? 2 : 1;  // tangential momentum component
+  // 2D loops over components and Gauss points stay rolled, their states in local memory: unrolled,
+  // the branches of all components and two forms of four points made 760 KB of code, far beyond
+  // the instruction cache (245 KB rolled; 64^2 order-7 run of 4 steps 435 -> 404 us).  1D unrolls its
+  // components: there the chain of one cell bounds the tile.
+  constexpr int kCU = (DIM == 1) ? C : 1;
+  // Products of the Gauss points on the integer units (ase_df_imul.cuh), where the tile has the
+  // warps to fill the FP64 pipe: the 1024^2 order-9 step 7393 -> 6466 us, the 65537-cell order-9
+  // residual 41.1 -> 39.0 us.  Tiles of up to 16 lines (4 warps of faces) and the 32-thread tiles are
+  // bound by latency and keep the FP64 instruction: with the integer form 64^2 runs were 7 - 9 %
+  // slower, 96^2 - 128^2 3 - 5 % faster and 160^2 1 - 6 % slower, those from 256^2 (28 lines) 8 - 14 % faster.
+  const bool ints = NT > 32 && (DIM == 1 || tt > 16);
 
   double* sW = smem;                       // [C][NB][NA]
   double* sQP = sW + C * NB * NA;          // [C][NB][NQ] value at xi = 0
@@ -573,7 +584,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         const Branch br = branch(sSn + bb * NSN + qa);
         if (R >= 5 && rough && pass == 0 && defer_item(br.m == 0, it, s_queue, &s_qn[0])) continue;
         if (pt < 0) {
-#pragma unroll
+#pragma unroll kCU
           for (int c = 0; c < C; ++c) {
             const double* v = sW + (c * NB + bb) * NA + qa + K;  // W_0 of this cell
             double out[2];
@@ -583,7 +594,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
           }
         } else {
           double* dst = pt ? sQM : sQP;
-#pragma unroll
+#pragma unroll kCU
           for (int c = 0; c < C; ++c) {
             const double* v = sW + (c * NB + bb) * NA + qa + K;
             double out[1];
@@ -654,40 +665,24 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       }
       // left state: cell f-1 (plus face); right: cell f (minus face)
       if constexpr (DIM == 2) {
-        if (!fixed) {
+#pragma unroll 1
+        for (int cs = 0; cs < 2 * C; ++cs) {
+          const int c = cs >> 1, side = cs & 1;
+          const int at = (c * NB + tb) * NQ + fa + side;  // line -K of the stencil
+          double out[G];
+          if (!fixed) {
+            tang_eval<R, G>((side == 0 ? sQP : sQM) + at + K * NQ, NQ, side == 0 ? bt[0] : bt[1], T, out);
+          } else if (pass == 0) {
+            fix_gauss<R, G, NQ>((side == 0 ? iQP : iQM) + at + K * NQ, comp_exp(c), out);
+          } else {
+            double v[2 * K + 1];
 #pragma unroll
-          for (int side = 0; side < 2; ++side)
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-              double out[G];
-              tang_eval<R, G>((side == 0 ? sQP : sQM) + (c * NB + tb + K) * NQ + fa + side, NQ, bt[side], T, out);
-#pragma unroll
-              for (int q = 0; q < G; ++q) st[side][q][c] = out[q];
-            }
-        } else if (pass == 0) {
-#pragma unroll
-          for (int c = 0; c < C; ++c) {
-#pragma unroll
-            for (int side = 0; side < 2; ++side) {
-              double out[G];
-              fix_gauss<R, G, NQ>((side == 0 ? iQP : iQM) + (c * NB + tb + K) * NQ + fa + side, comp_exp(c), out);
-#pragma unroll
-              for (int q = 0; q < G; ++q) st[side][q][c] = out[q];
-            }
+            for (int t = 0; t <= 2 * K; ++t)
+              v[t] = fix_to_double(fix_join((side == 0 ? iQP : iQM)[at + t * NQ]), comp_exp(c));
+            tang_eval<R, G>(v + K, 1, side == 0 ? bt[0] : bt[1], T, out);
           }
-        } else {
 #pragma unroll
-          for (int c = 0; c < C; ++c)
-#pragma unroll
-            for (int side = 0; side < 2; ++side) {
-              double v[2 * K + 1], out[G];
-#pragma unroll
-              for (int t = 0; t <= 2 * K; ++t)
-                v[t] = fix_to_double(fix_join((side == 0 ? iQP : iQM)[(c * NB + tb + t) * NQ + fa + side]), comp_exp(c));
-              tang_eval<R, G>(v + K, 1, bt[side], T, out);
-#pragma unroll
-              for (int q = 0; q < G; ++q) st[side][q][c] = out[q];
-            }
+          for (int q = 0; q < G; ++q) st[side][q][c] = out[q];
         }
       } else {
 #pragma unroll
@@ -704,11 +699,11 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       for (int c = 0; c < C; ++c) Fs[c] = 0.0;
       double ssum = 0.0;
       unsigned int nfb = 0u;
-#pragma unroll
+#pragma unroll 1
       for (int q = 0; q < G; ++q) {
         double sg;
-        nfb += lf_point_acc<C, NI, TI>(st[0][q], st[1][q], ca, cb, NB * NA, g.gm1, g.gg1, T.hgw[q], g.gm1_hgw[q],
-                                       Fs, sg) ? 1u : 0u;
+        nfb += lf_point_acc<C, NI, TI, (NT > 32)>(st[0][q], st[1][q], ca, cb, NB * NA, g.gm1, g.gg1, T.hgw[q],
+                                                  g.gm1_hgw[q], ints, Fs, sg) ? 1u : 0u;
         ssum += sg;
       }
       if (nfb) {
