@@ -354,7 +354,7 @@ const char* ase_df_last_error(const ase_df_ctx* c) { return c ? c->err : g_init_
 static cudaError_t sweep(ase_df_ctx* c, int dir, const double* W, const double* sx, const double* sy,
                          double* F, double* s_out, cudaStream_t s, double tfrac, int stage) {
   SweepArgs a;
-  if (stage >= 0 && looks_for_front(c->dim, c->g)) {
+  if (stage >= 0 && looks_for_front(c->dim, c->g, c->p.order)) {
     a.front = &c->st->front[stage > 0 ? stage - 1 : 0];
     if (stage == 1 || stage == 2) a.front_out = &c->st->front[stage];
   }
@@ -448,7 +448,7 @@ static cudaError_t combine(ase_df_ctx* c, int stage, const double* Wn, const dou
   r.dt_fixed = dt_fixed;
   r.stage = stage;
   r.tfrac = rk_tfrac(stage);
-  if (stage < 3 && looks_for_front(c->dim, c->g)) r.front_out = &c->st->front[stage];
+  if (stage < 3 && looks_for_front(c->dim, c->g, c->p.order)) r.front_out = &c->st->front[stage];
   r.pass = 1;
   if (small) return launch_combine_repair(c->g, a, r, s);
   ProfScope prof(c, s, 4);
@@ -471,7 +471,7 @@ static ase_df_status step_launches(ase_df_ctx* c, double* W, double* sx, double*
     sa.st = c->st;
     sa.inv_dx = c->inv_dx;
     sa.inv_dy = c->inv_dy;
-    if (looks_for_front(c->dim, c->g)) {
+    if (looks_for_front(c->dim, c->g, c->p.order)) {
       sa.sx = sx;
       sa.sy = sy;
     }
@@ -480,7 +480,7 @@ static ase_df_status step_launches(ase_df_ctx* c, double* W, double* sx, double*
       e = launch_max_speed(c->dim, c->g, sa, s);
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "max_speed");
-  } else if (looks_for_front(c->dim, c->g) && (e = launch_strength(c->g, sx, sy, c->st, s)) != cudaSuccess) {
+  } else if (looks_for_front(c->dim, c->g, c->p.order) && (e = launch_strength(c->g, sx, sy, c->st, s)) != cudaSuccess) {
     return cuda_fail(c, e, "strength scan");
   }
   const double dtf = (dt > 0.0) ? dt : 0.0;
@@ -507,7 +507,7 @@ ase_df_status ase_df_residual(ase_df_ctx* c, const double* W, const double* sx_i
     return fail(c, ASE_DF_E_INVAL, "sigma_out must not alias sigma_in");
   cudaStream_t s = (cudaStream_t)stream;
   c->last_stream = s;
-  cudaError_t e = looks_for_front(c->dim, c->g) ? launch_strength(c->g, sx_in, sy_in, c->st, s) : cudaSuccess;
+  cudaError_t e = looks_for_front(c->dim, c->g, c->p.order) ? launch_strength(c->g, sx_in, sy_in, c->st, s) : cudaSuccess;
   if (e == cudaSuccess) e = face_fluxes(c, W, sx_in, sy_in, sx_out, sy_out, s, 0);
   if (e != cudaSuccess) return cuda_fail(c, e, "residual sweep");
   e = combine(c, 0, W, W, L, 0.0, s);
@@ -743,7 +743,7 @@ ase_df_status ase_df_step_adjoint(ase_df_ctx* c, const double* W, const double* 
   double* s2by = (c->dim == 2) ? c->s2by : nullptr;
   cudaError_t e;
   // stages 1 and 2 of the forward step: W1, sigma1 (sxa, sya), W2, sigma2 (sxb, syb)
-  if (looks_for_front(c->dim, c->g) && (e = launch_strength(c->g, sx, sy, c->st, s)) != cudaSuccess)
+  if (looks_for_front(c->dim, c->g, c->p.order) && (e = launch_strength(c->g, sx, sy, c->st, s)) != cudaSuccess)
     return cuda_fail(c, e, "adjoint: strength scan");
   if ((e = face_fluxes(c, W, sx, sy, c->sxa, c->sya, s, 1)) != cudaSuccess) return cuda_fail(c, e, "adjoint: stage 1 sweep");
   if ((e = combine(c, 1, W, W, c->W1, dt, s, c->sxa, c->sya)) != cudaSuccess) return cuda_fail(c, e, "adjoint: stage 1 combine");

@@ -218,21 +218,26 @@ __device__ __forceinline__ bool lf_physical(double rhoL, double rhoR, const LfPr
   return pos_finite(rhoL) && pos_finite(rhoR) && pos_finite(s.pL) && pos_finite(s.pR);
 }
 
-// Flux and strength of a point from its states and their primitives.
-template <int C, int NI, int TI, bool INT = false>
-__device__ __forceinline__ void lf_flux(const double* a, const double* b, const LfPrims& s, bool ok, double gg1,
-                                        double w, double gw, double* Fs, double& sigma) {
+// What a point adds to its face: with its states a, b,
+//   w 2F_c = a_c alL + b_c alR + gw (ps on the normal momentum, pu on the energy).
+struct LfTerms {
+  double alL, alR, ps, pu;
+};
+
+// Terms and strength of a point from the primitives of its states.
+template <int C, bool INT = false>
+__device__ __forceinline__ LfTerms lf_terms(const LfPrims& s, bool ok, double gg1, double w, double& sigma) {
   const double irL = s.irL, irR = s.irR, unL = s.unL, unR = s.unR, utL = s.utL, utR = s.utR;
   const double pL = s.pL, pR = s.pR;
   const double c2L = lf_mul<INT>(lf_mul<INT>(gg1, pL), irL), c2R = lf_mul<INT>(lf_mul<INT>(gg1, pR), irR);
   const double icL = rsqrt_pos<INT>(c2L), icR = rsqrt_pos<INT>(c2R);
   // lambda = max(|u_n| + c) with c = c^2 / c
   const double lam = max_nonneg(fma(c2L, icL, fabs(unL)), fma(c2R, icR, fabs(unR)));
-  const double alL = lf_mulz<INT>(unL + lam, w), alR = lf_mulz<INT>(unR - lam, w);
-  Fs[0] = fma(a[0], alL, fma(b[0], alR, Fs[0]));
-  Fs[NI] = fma(a[NI], alL, fma(b[NI], alR, fma(gw, pL + pR, Fs[NI])));
-  if (C == 4) Fs[TI] = fma(a[TI], alL, fma(b[TI], alR, Fs[TI]));
-  Fs[C - 1] = fma(a[C - 1], alL, fma(b[C - 1], alR, fma(gw, fma(unL, pL, lf_mulz<INT>(unR, pR)), Fs[C - 1])));
+  LfTerms t;
+  t.alL = lf_mulz<INT>(unL + lam, w);
+  t.alR = lf_mulz<INT>(unR - lam, w);
+  t.ps = pL + pR;
+  t.pu = fma(unL, pL, lf_mulz<INT>(unR, pR));
   if (ok) {
     // sigma = |dp| (1/p_l + 1/p_r) + (dMa_n)^2 + (dMa_t)^2, Ma = u / c
     const double dmn = fma(unL, icL, -lf_mulz<INT>(unR, icR));
@@ -247,32 +252,40 @@ __device__ __forceinline__ void lf_flux(const double* a, const double* b, const 
   } else {
     sigma = kSigmaBig;
   }
+  return t;
 }
 
-// ints (with INT): the products on the integer units.  They are there for states within imul_pos /
-// imul_any, which bound every operand of a point; others, non-physical ones among them, take the
-// FP64 unit.
-template <int C, int NI, int TI, bool INT = false>
-__device__ __forceinline__ bool lf_point_acc(const double* qa, const double* qb, const double* ca,
-                                             const double* cb, int cs, double gm1, double gg1, double w,
-                                             double gw, bool ints, double* Fs, double& sigma) {
-  if (INT) {
-    bool in = ints && imul_pos(qa[0]) && imul_pos(qb[0]) && imul_pos(gg1);
-#pragma unroll
-    for (int c = 1; c < C - 1; ++c) in = in && imul_any(qa[c]) && imul_any(qb[c]);
-    if (in) {
-      const LfPrims s = lf_primitives<C, NI, TI, true>(qa, qb);
-      if (imul_pos(s.pL) && imul_pos(s.pR)) {
-        lf_flux<C, NI, TI, true>(qa, qb, s, true, gg1, w, gw, Fs, sigma);
-        return false;
-      }
-    }
-  }
-  double a[C], b[C];
+// Component c of a point added to its Gauss sum F.
+template <int C, int NI>
+__device__ __forceinline__ double lf_add(int c, double a, double b, const LfTerms& t, double gw, double F) {
+  const double base = c == NI ? fma(gw, t.ps, F) : c == C - 1 ? fma(gw, t.pu, F) : F;
+  return fma(a, t.alL, fma(b, t.alR, base));
+}
+
+// States a, b of a point (qa, qb, or the cell averages), its terms and strength; whether it took
+// the cell averages.  ints (with INT): the products on the integer units.  They are there for states
+// within imul_pos / imul_any, which bound every operand of a point; others, non-physical ones among
+// them, take the FP64 unit.
+template <int C, int NI, int TI, bool INT>
+__device__ __forceinline__ bool lf_point_terms(const double* qa, const double* qb, const double* ca, const double* cb,
+                                               int cs, double gg1, double w, bool ints, double* a, double* b,
+                                               LfTerms& t, double& sigma) {
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     a[c] = qa[c];
     b[c] = qb[c];
+  }
+  if (INT) {
+    bool in = ints && imul_pos(a[0]) && imul_pos(b[0]) && imul_pos(gg1);
+#pragma unroll
+    for (int c = 1; c < C - 1; ++c) in = in && imul_any(a[c]) && imul_any(b[c]);
+    if (in) {
+      const LfPrims s = lf_primitives<C, NI, TI, true>(a, b);
+      if (imul_pos(s.pL) && imul_pos(s.pR)) {
+        t = lf_terms<C, true>(s, true, gg1, w, sigma);
+        return false;
+      }
+    }
   }
   LfPrims s = lf_primitives<C, NI, TI>(a, b);
   const bool ok = lf_physical(a[0], b[0], s);
@@ -284,8 +297,20 @@ __device__ __forceinline__ bool lf_point_acc(const double* qa, const double* qb,
     }
     s = lf_primitives<C, NI, TI>(a, b);
   }
-  lf_flux<C, NI, TI>(a, b, s, ok, gg1, w, gw, Fs, sigma);
+  t = lf_terms<C>(s, ok, gg1, w, sigma);
   return !ok;
+}
+
+template <int C, int NI, int TI, bool INT = false>
+__device__ __forceinline__ bool lf_point_acc(const double* qa, const double* qb, const double* ca,
+                                             const double* cb, int cs, double gm1, double gg1, double w,
+                                             double gw, bool ints, double* Fs, double& sigma) {
+  double a[C], b[C];
+  LfTerms t;
+  const bool first = lf_point_terms<C, NI, TI, INT>(qa, qb, ca, cb, cs, gg1, w, ints, a, b, t, sigma);
+#pragma unroll
+  for (int c = 0; c < C; ++c) Fs[c] = lf_add<C, NI>(c, a[c], b[c], t, gw, Fs[c]);
+  return first;
 }
 
 // The flux of one point as 2F = F_l + F_r - lambda (q_r - q_l), and sigma (lf_point_acc with

@@ -223,9 +223,9 @@ cudaError_t launch_combine(int dim, const GridInfo& g, const CombineArgs& a, cud
 cudaError_t launch_max_speed(int dim, const GridInfo& g, const SpeedArgs& a, cudaStream_t s);
 // Single 2D problems below this many cells keep to FP64: a step is bound by its chain of launches
 // there, and looking for a front costs what the fixed-point sweep gains.
-constexpr long long kFrontCells = 128 * 128;
-inline bool looks_for_front(int dim, const GridInfo& g) {
-  return dim == 2 && (long long)g.nx * g.ny >= kFrontCells;
+constexpr long long kFrontCells = 128 * 128, kFrontCells3 = 200 * 200;
+inline bool looks_for_front(int dim, const GridInfo& g, int order) {
+  return dim == 2 && (long long)g.nx * g.ny >= (order == 3 ? kFrontCells3 : kFrontCells);
 }
 // front[0] of the status word from the strengths a 2D stage consumes.
 cudaError_t launch_strength(const GridInfo& g, const double* sx, const double* sy, DevState* st, cudaStream_t s);

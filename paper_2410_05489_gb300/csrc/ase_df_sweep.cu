@@ -89,6 +89,8 @@ cudaError_t launch(const GridInfo& g, const SweepArgs& a, const Tables& t, cudaS
         p = p8;
         tiles = tiles8;
       }
+      // tiles of at most 16 lines: several threads a face (sweep_tile)
+      if ((m + p.nb_lo - 1) / p.nb_lo <= 16) return launch_grid<R, DIM, DIR, 16, true>(g, a, t, s, dim3((unsigned)tiles), p);
       return launch_grid<R, DIM, DIR, TT, true>(g, a, t, s, dim3((unsigned)tiles), p);
     }
     if (cols > 0x7fffffffLL || q > 65535) return cudaErrorInvalidConfiguration;

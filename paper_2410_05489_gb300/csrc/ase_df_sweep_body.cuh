@@ -232,7 +232,11 @@ struct Tile {
   static constexpr size_t smem_doubles = queue_offset + ((size_t)QCAP + 2 + 1) / 2;
   // 2D sweeps, after the queue: a flag (2 ints) and 8 ints per warp (TileSpan)
   static constexpr size_t span_offset = smem_doubles;
-  static constexpr size_t sweep_doubles = smem_doubles + (DIM == 2 ? 1 + (size_t)(NT / 32) * 4 : 0);
+  static constexpr size_t split_offset = smem_doubles + (DIM == 2 ? 1 + (size_t)(NT / 32) * 4 : 0);
+  // 2D tiles of 16 lines, last: the states [2][G][C] and terms [5][G] of every face and the
+  // branches (5 words) of its columns (sweep_tile)
+  static constexpr bool split = DIM == 2 && TT == 16;
+  static constexpr size_t sweep_doubles = split_offset + (split ? (size_t)(2 * C + 5) * G * TN * TT + 5 * NQ * TT : 0);
 };
 
 // Quotient and remainder by a tile's run-time line count n (at most 127) of an index below 2^13, by
@@ -395,13 +399,13 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   // the branches of all components and two forms of four points made 760 KB of code, far beyond
   // the instruction cache (245 KB rolled; 64^2 order-7 run of 4 steps 435 -> 404 us).  1D unrolls its
   // components: there the chain of one cell bounds the tile.
-  constexpr int kCU = (DIM == 1) ? C : 1;
+  constexpr int kCU = (DIM == 1) ? C : 1, kLU = TL::split ? 1 : C;
   // Products of the Gauss points on the integer units (ase_df_imul.cuh), where the tile has the
   // warps to fill the FP64 pipe: the 1024^2 order-9 step 7393 -> 6466 us, the 65537-cell order-9
-  // residual 41.1 -> 39.0 us.  Tiles of up to 16 lines (4 warps of faces) and the 32-thread tiles are
-  // bound by latency and keep the FP64 instruction: with the integer form 64^2 runs were 7 - 9 %
-  // slower, 96^2 - 128^2 3 - 5 % faster and 160^2 1 - 6 % slower, those from 256^2 (28 lines) 8 - 14 % faster.
-  const bool ints = NT > 32 && (DIM == 1 || tt > 16);
+  // residual 41.1 -> 39.0 us.  The 32-thread tiles and those of up to 8 lines (two CTAs of a few warps'
+  // work on an SM) are bound by latency and keep the FP64 instruction: 64^2 order-7 runs 324 us, 332 with
+  // the integer form; 128^2 ones 619 and 577 us.
+  const bool ints = NT > 32 && (!TL::split || tt > 8);
 
   double* sW = smem;                       // [C][NB][NA]
   double* sQP = sW + C * NB * NA;          // [C][NB][NQ] value at xi = 0
@@ -439,7 +443,11 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   const bool inside = DIM == 2 && a0 - 1 - K >= 0 && a0 + TN - 1 + K < n && b0 - KT >= 0 && b0 + tt + KT <= mlin;
   // cell averages: cells a0-1-K .. a0+TN-1+K, lines b0-KT .. b0+tt+KT-1
   TileSpan span;
-  for (int idx = tid; idx < nb * NA; idx += NT) {
+  // (16-line tiles: one component of a cell per thread, which loads one value instead of four in turn)
+  const int staged = nb * NA;
+  for (int k = tid; k < (TL::split ? C * staged : staged); k += NT) {
+    const int c0 = TL::split ? (k >= staged) + (k >= 2 * staged) + (k >= 3 * staged) : 0;
+    const int cn = TL::split ? c0 + 1 : C, idx = k - c0 * staged;
     int bb, aa;
     if (DIR == 0) { aa = idx % NA; bb = idx / NA; }
     else dnb.split(idx, aa, bb);
@@ -447,8 +455,8 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
     double* dst = sW + bb * NA + aa;
     if (inside) {
       const double* src = args.W + (size_t)b * stb + (size_t)a * sta;
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
+#pragma unroll kLU
+      for (int c = c0; c < cn; ++c) {
         const double v = __ldg(src + (size_t)c * g.nx * g.ny);
         dst[c * NB * NA] = v;
         if (DIM == 2) span.add(c, C - 1, v);
@@ -456,7 +464,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
     } else {
       const int i = (DIR == 0) ? a : b, j = (DIR == 0) ? b : a;
 #pragma unroll 1
-      for (int c = 0; c < C; ++c) {
+      for (int c = c0; c < cn; ++c) {
         const double v = fetch_w(g, args.W, c, i, j, ts);
         dst[c * NB * NA] = v;
         if (DIM == 2) span.add(c, C - 1, v);
@@ -566,12 +574,16 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   }
   if (!fixed) {
     // FP64: the end cells come last in the work list and evaluate one point; fallback cells are
-    // deferred (defer_item) and done in a second pass
+    // deferred (defer_item) and done in a second pass.  A 16-line tile without a branch choice
+    // gives each component of a cell a thread.
+    const bool comps = TL::split && !rough;
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
-      const int count = (pass == 0) ? NQ * nb : (int)s_qn[0];
+      const int cells = NQ * nb;
+      const int count = (pass == 0) ? (comps ? C * cells : cells) : (int)s_qn[0];
       for (int k = tid; k < count; k += NT) {
-        const int it = (pass == 0) ? k : s_queue[k];
+        const int c0 = comps ? (k >= cells) + (k >= 2 * cells) + (k >= 3 * cells) : 0, cn = comps ? c0 + 1 : C;
+        const int it = (pass == 0) ? k - c0 * cells : s_queue[k];
         int qa, bb, pt;  // pt -1: an interior cell, both points; 0 / 1: an end cell, one point
         if (it < (NQ - 2) * nb) {
           if (DIR == 0) { qa = 1 + it % (NQ - 2); bb = it / (NQ - 2); }
@@ -585,7 +597,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         if (R >= 5 && rough && pass == 0 && defer_item(br.m == 0, it, s_queue, &s_qn[0])) continue;
         if (pt < 0) {
 #pragma unroll kCU
-          for (int c = 0; c < C; ++c) {
+          for (int c = c0; c < cn; ++c) {
             const double* v = sW + (c * NB + bb) * NA + qa + K;  // W_0 of this cell
             double out[2];
             recon_eval<R, 2>(v, 1, br, T, 0, out);
@@ -595,7 +607,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         } else {
           double* dst = pt ? sQM : sQP;
 #pragma unroll kCU
-          for (int c = 0; c < C; ++c) {
+          for (int c = c0; c < cn; ++c) {
             const double* v = sW + (c * NB + bb) * NA + qa + K;
             double out[1];
             recon_eval<R, 1>(v, 1, br, T, pt, out);
@@ -631,9 +643,126 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
     }
   }
 
+  // Gauss-point values of component cs / 2 of the state on side cs % 2 of a face, its branch bt;
+  // fixed point: in FP64 from the limbs where a side of the face has another branch (lin: none has)
+  auto tang_point = [&](int cs, int fa, int tb, const Branch& bt, bool lin, double* out) {
+    const int c = cs >> 1, side = cs & 1;
+    const int at = (c * NB + tb) * NQ + fa + side;  // line -K of the stencil
+    if (!fixed) {
+      tang_eval<R, G>((side == 0 ? sQP : sQM) + at + K * NQ, NQ, bt, T, out);
+    } else if (lin) {
+      fix_gauss<R, G, NQ>((side == 0 ? iQP : iQM) + at + K * NQ, comp_exp(c), out);
+    } else {
+      double v[2 * K + 1];
+#pragma unroll
+      for (int t = 0; t <= 2 * K; ++t)
+        v[t] = fix_to_double(fix_join((side == 0 ? iQP : iQM)[at + t * NQ]), comp_exp(c));
+      tang_eval<R, G>(v + K, 1, bt, T, out);
+    }
+  };
   // ---- phase 2: faces ----
   // 2D: faces with a fallback tangential reconstruction on either side (fixed point: with any but
   // the order-R linear one) are deferred.
+  if constexpr (TL::split) {
+    // Tiles of up to 16 lines, on grids that give an SM one or two of them: a face per thread would
+    // leave half or more of the CTA idle while a quarter of the SM's FP64 unit works on chains of some
+    // 100 dependent instructions.  So (component, side) pairs of a face, then its Gauss points, then
+    // the components of its sums go to threads of their own, in the same arithmetic and order.
+    constexpr int NF = TN * TT;
+    double* sP = smem + TL::split_offset;  // [2][G][C][NF] states
+    double* sX = sP + 2 * G * C * NF;      // [G][5][NF]: alL, alR, ps, pu, strength
+    static_assert(sizeof(Branch) == 5 * sizeof(double), "sB");
+    Branch* sB = reinterpret_cast<Branch*>(sX + 5 * G * NF);  // [TT][NQ] branches of the columns
+    const int faces = TN * tt;
+    const LineDiv dtt(tt);
+    auto face_of = [&](int it, int& fa, int& tb) {
+      if (DIR == 0) { fa = it % TN; tb = it / TN; }
+      else dtt.split(it, fa, tb);
+      return a0 + fa <= n && b0 + tb < mlin;
+    };
+    if (rough) {
+      for (int it = tid; it < NQ * tt; it += NT) sB[it] = select_branch<R>(sSt + (it % NQ) * NST + it / NQ, g.thres);
+      __syncthreads();
+    }
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+      const int nf = (pass == 0) ? faces : (int)s_qn[1];
+      for (int k = tid; k < 2 * C * nf; k += NT) {
+        int cs = 0, kf = k;
+        while (kf >= nf) { kf -= nf; ++cs; }
+        const int it = (pass == 0) ? kf : s_queue[kf];
+        int fa, tb;
+        if (!face_of(it, fa, tb)) continue;
+        Branch bt = linear_branch<R>();
+        if (rough) bt = sB[tb * NQ + fa + (cs & 1)];
+        if (rough && pass == 0) {
+          const int m2 = sB[tb * NQ + fa + 1 - (cs & 1)].m;  // the other side's
+          const bool later = fixed ? bt.m != R || m2 != R : R >= 5 && (bt.m == 0 || m2 == 0);
+          if (defer_item(later && cs == 0, it, s_queue, &s_qn[1]) || later) continue;
+        }
+        if (counting && cs < 2) {
+          atomicAdd(&hist_s[branch_slot(select_branch<R>(sSn + (tb + KT) * NSN + fa + cs, g.thres).m)], 1u);
+          atomicAdd(&hist_s[branch_slot(bt.m)], 1u);
+        }
+        double out[G];
+        tang_point(cs, fa, tb, bt, pass == 0, out);
+#pragma unroll
+        for (int q = 0; q < G; ++q) sP[(((cs & 1) * G + q) * C + (cs >> 1)) * NF + it] = out[q];
+      }
+      __syncthreads();
+      if (s_qn[1] == 0u) break;
+    }
+    for (int k = tid; k < G * faces; k += NT) {
+      int q = 0, it = k;
+      while (it >= faces) { it -= faces; ++q; }
+      int fa, tb;
+      if (!face_of(it, fa, tb)) continue;
+      double qa[C], qb[C], a[C], b[C], sg;
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        qa[c] = sP[(q * C + c) * NF + it];
+        qb[c] = sP[((G + q) * C + c) * NF + it];
+      }
+      const double* ca = sW + (tb + KT) * NA + fa + K;
+      LfTerms t;
+      if (lf_point_terms<C, NI, TI, true>(qa, qb, ca, ca + 1, NB * NA, g.gg1, T.hgw[q], ints, a, b, t, sg)) {
+        atomicOr(&args.st->flags, 0x2u);
+        if (counting) atomicAdd(&hist_s[kBranchSlots - 1], 1u);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          sP[(q * C + c) * NF + it] = a[c];
+          sP[((G + q) * C + c) * NF + it] = b[c];
+        }
+      }
+      const double x[5] = {t.alL, t.alR, t.ps, t.pu, sg};
+#pragma unroll
+      for (int j = 0; j < 5; ++j) sX[(q * 5 + j) * NF + it] = x[j];
+    }
+    __syncthreads();
+    for (int k = tid; k < (C + 1) * faces; k += NT) {
+      int c = 0, it = k;
+      while (it >= faces) { it -= faces; ++c; }
+      int fa, tb;
+      if (!face_of(it, fa, tb)) continue;
+      const int f = a0 + fa, b = b0 + tb;
+      double sum = 0.0;
+#pragma unroll
+      for (int q = 0; q < G; ++q) {
+        const double* x = sX + q * 5 * NF + it;
+        if (c == C) sum += x[4 * NF];
+        else sum = lf_add<C, NI>(c, sP[(q * C + c) * NF + it], sP[((G + q) * C + c) * NF + it],
+                                 LfTerms{x[0], x[NF], x[2 * NF], x[3 * NF]}, g.gm1_hgw[q], sum);
+      }
+      if (c < C) {
+        if (DIR == 0) args.F[((size_t)c * g.ny + b) * (g.nx + 1) + f] = sum;
+        else args.F[((size_t)c * (g.ny + 1) + f) * g.nx + b] = sum;
+      } else {
+        const double sface = (G == 1) ? sum : sum * (1.0 / G);
+        if (args.front_out != nullptr && is_front(sface, limit)) *args.front_out = 1u;
+        args.s_out[(DIR == 0) ? (size_t)b * (g.nx + 1) + f : (size_t)f * g.nx + b] = sface;
+      }
+    }
+  } else {
   const LineDiv dtt(tt);
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
@@ -667,22 +796,10 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       if constexpr (DIM == 2) {
 #pragma unroll 1
         for (int cs = 0; cs < 2 * C; ++cs) {
-          const int c = cs >> 1, side = cs & 1;
-          const int at = (c * NB + tb) * NQ + fa + side;  // line -K of the stencil
           double out[G];
-          if (!fixed) {
-            tang_eval<R, G>((side == 0 ? sQP : sQM) + at + K * NQ, NQ, side == 0 ? bt[0] : bt[1], T, out);
-          } else if (pass == 0) {
-            fix_gauss<R, G, NQ>((side == 0 ? iQP : iQM) + at + K * NQ, comp_exp(c), out);
-          } else {
-            double v[2 * K + 1];
+          tang_point(cs, fa, tb, (cs & 1) == 0 ? bt[0] : bt[1], pass == 0, out);
 #pragma unroll
-            for (int t = 0; t <= 2 * K; ++t)
-              v[t] = fix_to_double(fix_join((side == 0 ? iQP : iQM)[at + t * NQ]), comp_exp(c));
-            tang_eval<R, G>(v + K, 1, side == 0 ? bt[0] : bt[1], T, out);
-          }
-#pragma unroll
-          for (int q = 0; q < G; ++q) st[side][q][c] = out[q];
+          for (int q = 0; q < G; ++q) st[cs & 1][q][cs >> 1] = out[q];
         }
       } else {
 #pragma unroll
@@ -725,6 +842,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
     if (DIM == 1 || pass == 1) break;
     __syncthreads();  // the queue is complete
     if (s_qn[1] == 0u) break;
+  }
   }
   if (counting) {
     __syncthreads();
