@@ -258,13 +258,13 @@ __device__ __forceinline__ void sigma_vjp(const Branch& br, const double* ab, do
 // constant sigma 1e30), sets ab / bb to the adjoints of the states a / b.  |x| and max take
 // the symmetric subgradient near their kinks (reading G23, kKink).
 // s = lf_primitives(a, b).
-template <int C, int NI, int TI>
+template <int C, int NI, int TI, bool INT = false>
 __device__ __forceinline__ void lf_point_vjp(const double* a, const double* b, const LfPrims& s, double gm1,
                                              double gg1, const double* F2b, double sb, bool physical, double* ab,
                                              double* bb) {
-  const double c2L = (gg1 * s.pL) * s.irL, c2R = (gg1 * s.pR) * s.irR;
-  const double icL = rsqrt_pos(c2L), icR = rsqrt_pos(c2R);
-  const double cL = c2L * icL, cR = c2R * icR;
+  const double c2L = lf_mul<INT>(lf_mul<INT>(gg1, s.pL), s.irL), c2R = lf_mul<INT>(lf_mul<INT>(gg1, s.pR), s.irR);
+  const double icL = rsqrt_pos<INT>(c2L), icR = rsqrt_pos<INT>(c2R);
+  const double cL = lf_mul<INT>(c2L, icL), cR = lf_mul<INT>(c2R, icR);
   const double sL = fabs(s.unL) + cL, sR = fabs(s.unR) + cR;
   const double lam = fmax(sL, sR);
   // direct terms of 2F and the adjoints of u, p', lambda
@@ -289,14 +289,14 @@ __device__ __forceinline__ void lf_point_vjp(const double* a, const double* b, c
   uRb = fma(sRb, dabs(s.unR, cR), uRb);
   double cLb = sLb, cRb = sRb, icLb = 0.0, icRb = 0.0, irLb = 0.0, irRb = 0.0, wLb = 0.0, wRb = 0.0;
   if (physical && sb != 0.0) {
-    const double dmn = fma(s.unL, icL, -s.unR * icR);
+    const double dmn = fma(s.unL, icL, -lf_mulz<INT>(s.unR, icR));
     const double gn = 2.0 * sb * dmn;
     uLb = fma(gn, icL, uLb);
     uRb = fma(-gn, icR, uRb);
     icLb = fma(gn, s.unL, icLb);
     icRb = fma(-gn, s.unR, icRb);
     if (C == 4) {
-      const double dmt = fma(s.utL, icL, -s.utR * icR);
+      const double dmt = fma(s.utL, icL, -lf_mulz<INT>(s.utR, icR));
       const double gt = 2.0 * sb * dmt;
       wLb = gt * icL;
       wRb = -gt * icR;
@@ -304,7 +304,7 @@ __device__ __forceinline__ void lf_point_vjp(const double* a, const double* b, c
       icRb = fma(-gt, s.utR, icRb);
     }
     const double dp = s.pL - s.pR;
-    const double S = fma(s.irL * icL, icL, s.irR * icR * icR);
+    const double S = fma(lf_mul<INT>(s.irL, icL), icL, lf_mul<INT>(lf_mul<INT>(s.irR, icR), icR));
     const double gp = sb * gg1 * dabs(dp, s.pL + s.pR) * S;
     pLb += gp;
     pRb -= gp;
@@ -316,8 +316,8 @@ __device__ __forceinline__ void lf_point_vjp(const double* a, const double* b, c
   }
   // c = sqrt(c^2), ic = 1 / sqrt(c^2): dc/dc^2 = ic / 2, d ic / dc^2 = -ic^3 / 2;
   // c^2 = gamma (gamma-1) p' / rho
-  const double c2Lb = 0.5 * icL * fma(-icLb, icL * icL, cLb);
-  const double c2Rb = 0.5 * icR * fma(-icRb, icR * icR, cRb);
+  const double c2Lb = 0.5 * icL * fma(-icLb, lf_mul<INT>(icL, icL), cLb);
+  const double c2Rb = 0.5 * icR * fma(-icRb, lf_mul<INT>(icR, icR), cRb);
   pLb = fma(c2Lb * gg1, s.irL, pLb);
   pRb = fma(c2Rb * gg1, s.irR, pRb);
   irLb = fma(c2Lb * gg1, s.pL, irLb);
@@ -398,7 +398,11 @@ __device__ __forceinline__ int face_preimages(int e, int n, int bl, int bh, int 
 // at 168 registers), three at order 9 (its 64 KB of shared memory per CTA allows no more);
 // 1D: 256 faces per CTA of 256 threads.  Phase A (per face) recomputes the two states at
 // each Gauss point and writes their adjoints to shared memory; phase B (per face and side)
-// takes them back through the tangential reconstruction.
+// takes them back through the tangential reconstruction.  The loops over components of the recomputed
+// forward are rolled (443 -> 320 KB of code at order 7), and the 26 products of a point's primitives and
+// of its VJP that no cotangent enters run on the integer units (ase_df_imul.cuh), to the bit:
+// residual adjoint at order 7, 256^2 346 -> 334 us, 400^2 795 -> 767; order 9, 256^2 475 -> 461.  With the FP64
+// instruction and phase B rolled too it was 353 us.
 template <int R, int DIM>
 struct AdjShape {
   static constexpr int TN = (DIM == 2) ? 8 : 256;
@@ -476,7 +480,7 @@ adj_face_kernel(const GridInfo g, const SweepArgs args, const AdjArgs aa, const 
   for (int it = tid; it < NQ * NB; it += NT) {
     const int qa = it % NQ, bb = it / NQ;
     const Branch br = select_branch<R>(sSn + bb * NSN + qa, g.thres);
-#pragma unroll
+#pragma unroll 1
     for (int c = 0; c < C; ++c) {
       const double* v = sW + (c * NB + bb) * NA + qa + K;
       double out[2];
@@ -525,13 +529,13 @@ adj_face_kernel(const GridInfo g, const SweepArgs args, const AdjArgs aa, const 
 #pragma unroll 1
       for (int q = 0; q < G; ++q) {
         double st[2][C];
-#pragma unroll
+#pragma unroll 1
         for (int side = 0; side < 2; ++side) {
           const int qa = fa + side;
           const double* Q = side == 0 ? sQP : sQM;
           if (DIM == 2) {
             const Branch bt = select_branch<R>(sSt + qa * NST + tb, g.thres);
-#pragma unroll
+#pragma unroll 1
             for (int c = 0; c < C; ++c) {
               double out[1];
               recon_eval<R, 1>(Q + (c * NB + tb + K) * NQ + qa, NQ, bt, T, 2 + q, out);
@@ -546,12 +550,22 @@ adj_face_kernel(const GridInfo g, const SweepArgs args, const AdjArgs aa, const 
         const double hw = T.hgw[q];
 #pragma unroll
         for (int c = 0; c < C; ++c) F2b[c] = hw * Fb[c];
-        const LfPrims pr = lf_primitives<C, NI, TI>(st[0], st[1]);
+        bool in = imul_pos(st[0][0]) && imul_pos(st[1][0]) && imul_pos(g.gg1);
+#pragma unroll
+        for (int c = 1; c < C - 1; ++c) in = in && imul_any(st[0][c]) && imul_any(st[1][c]);
+        LfPrims pr;
+        if (in) {
+          pr = lf_primitives<C, NI, TI, true>(st[0], st[1]);
+          in = imul_pos(pr.pL) && imul_pos(pr.pR);
+        } else {
+          pr = lf_primitives<C, NI, TI>(st[0], st[1]);
+        }
         double* out0 = sStb + (size_t)(q * C) * NT + it;        // side 0, point q, component 0
         double* out1 = sStb + (size_t)((G + q) * C) * NT + it;  // side 1
         double ab[C], bb[C];
         if (lf_physical(st[0][0], st[1][0], pr)) {
-          lf_point_vjp<C, NI, TI>(st[0], st[1], pr, g.gm1, g.gg1, F2b, sbar, true, ab, bb);
+          if (in) lf_point_vjp<C, NI, TI, true>(st[0], st[1], pr, g.gm1, g.gg1, F2b, sbar, true, ab, bb);
+          else lf_point_vjp<C, NI, TI>(st[0], st[1], pr, g.gm1, g.gg1, F2b, sbar, true, ab, bb);
 #pragma unroll
           for (int c = 0; c < C; ++c) {
             out0[c * NT] = ab[c];
