@@ -93,7 +93,9 @@ __device__ __forceinline__ double rsqrt_pos(double x) {
 }
 
 // cell index 0..n-1 of a (ghost) cell; a reflecting wall mirrors about its face (the
-// ghost layers reach at most k+1 <= n cells deep, which the context validates); the wall
+// ghost layers reach at most k+1 <= n cells deep, which the context validates; a tile that
+// overhangs a grid of few cells stages cells beyond them, which no face reads, and those stop at
+// the far end instead of leaving the array); the wall
 // part of a BC_WALL_AFTER boundary mirrors too (its fixed part is handled by the callers)
 __device__ __forceinline__ int wrap_or_clamp(int i, int n, int bc_lo, int bc_hi) {
   if (i < 0) {
@@ -103,7 +105,7 @@ __device__ __forceinline__ int wrap_or_clamp(int i, int n, int bc_lo, int bc_hi)
   }
   if (i >= n) {
     if (bc_hi == BC_PERIODIC) return i % n;
-    if (bc_hi == BC_REFLECT) return 2 * n - 1 - i;
+    if (bc_hi == BC_REFLECT) return max(2 * n - 1 - i, 0);
     return n - 1;
   }
   return i;
@@ -118,7 +120,7 @@ __device__ __forceinline__ int face_map(int f, int n, int bc_lo, int bc_hi) {
     return 0;
   }
   if (bc_hi == BC_PERIODIC) return f % n;
-  if (bc_hi == BC_REFLECT) return 2 * n - f;
+  if (bc_hi == BC_REFLECT) return max(2 * n - f, 0);
   return n;
 }
 
