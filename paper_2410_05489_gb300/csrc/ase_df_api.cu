@@ -355,8 +355,8 @@ static cudaError_t sweep(ase_df_ctx* c, int dir, const double* W, const double* 
                          double* F, double* s_out, cudaStream_t s, double tfrac, int stage) {
   SweepArgs a;
   if (stage >= 0 && looks_for_front(c->dim, c->g, c->p.order)) {
-    a.front = &c->st->front[stage > 0 ? stage - 1 : 0];
-    if (stage == 1 || stage == 2) a.front_out = &c->st->front[stage];
+    a.front = c->st->front[stage > 0 ? stage - 1 : 0];
+    if (stage == 1 || stage == 2) a.front_out = &c->st->front[stage][dir];
   }
   a.tfrac = tfrac;
   a.W = W;
@@ -448,7 +448,7 @@ static cudaError_t combine(ase_df_ctx* c, int stage, const double* Wn, const dou
   r.dt_fixed = dt_fixed;
   r.stage = stage;
   r.tfrac = rk_tfrac(stage);
-  if (stage < 3 && looks_for_front(c->dim, c->g, c->p.order)) r.front_out = &c->st->front[stage];
+  if (stage < 3 && looks_for_front(c->dim, c->g, c->p.order)) r.front_out = c->st->front[stage];
   r.pass = 1;
   if (small) return launch_combine_repair(c->g, a, r, s);
   ProfScope prof(c, s, 4);

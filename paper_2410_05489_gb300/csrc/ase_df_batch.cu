@@ -129,8 +129,8 @@ batch_sweep_kernel(const BatchProblem* __restrict__ probs, const int4* __restric
     a.F = (DIR == 0) ? P.Fx + pb.fx_off : P.Fy + pb.fy_off;
     a.s_out = (DIR == 0) ? sp.sxout : sp.syout;
     a.st = states + w.x;
-    if (stage > 0) a.front = &a.st->front[stage - 1];  // read for 2D problems only
-    if (stage == 1 || stage == 2) a.front_out = &a.st->front[stage];
+    if (stage > 0) a.front = a.st->front[stage - 1];  // read for 2D problems only
+    if (stage == 1 || stage == 2) a.front_out = &a.st->front[stage][DIR];
     if (DIR == 0 && w.y == 0 && w.z == 0 && threadIdx.x <= kRepairPasses) {
       a.st->cnt[threadIdx.x] = 0u;  // repair counters of this problem's stage
       a.st->rbad[threadIdx.x] = 0u;
@@ -205,7 +205,7 @@ __device__ __forceinline__ RepairArgs repair_args(const BatchPtrs& P, const Batc
   r.dt_fixed = 0.0;
   r.stage = stage;
   r.pass = pass;
-  if (stage < 3) r.front_out = &st->front[stage];
+  if (stage < 3) r.front_out = st->front[stage];
   return r;
 }
 
@@ -246,8 +246,8 @@ __global__ void __launch_bounds__(256) batch_max_speed_kernel(const BatchProblem
     // the same share of the strengths, the last chunk also the ny (nx) entries past the cell count
     const size_t ncell = (size_t)pb.g.nx * pb.g.ny;
     const bool tail = (size_t)ch.z == ncell;
-    front_range(P.sx + pb.sx_off, first, tail ? ncell + pb.g.ny : (size_t)ch.z, blockDim.x, pb.g.thres, &a.st->front[0]);
-    front_range(P.sy + pb.sy_off, first, tail ? ncell + pb.g.nx : (size_t)ch.z, blockDim.x, pb.g.thres, &a.st->front[0]);
+    front_range(P.sx + pb.sx_off, first, tail ? ncell + pb.g.ny : (size_t)ch.z, blockDim.x, pb.g.thres, &a.st->front[0][0]);
+    front_range(P.sy + pb.sy_off, first, tail ? ncell + pb.g.nx : (size_t)ch.z, blockDim.x, pb.g.thres, &a.st->front[0][1]);
   }
 }
 

@@ -118,8 +118,8 @@ __global__ void __launch_bounds__(256) max_speed_kernel(const GridInfo g, const 
   const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
   max_speed_range<DIM>(g, a, first, (size_t)g.nx * g.ny, stride);
   if (DIM == 2 && a.sx != nullptr) {
-    front_range(a.sx, first, (size_t)g.ny * (g.nx + 1), stride, g.thres, &a.st->front[0]);
-    front_range(a.sy, first, (size_t)(g.ny + 1) * g.nx, stride, g.thres, &a.st->front[0]);
+    front_range(a.sx, first, (size_t)g.ny * (g.nx + 1), stride, g.thres, &a.st->front[0][0]);
+    front_range(a.sy, first, (size_t)(g.ny + 1) * g.nx, stride, g.thres, &a.st->front[0][1]);
   }
 }
 
@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(256) strength_kernel(const double* __restrict_
                                                        const double* __restrict__ sy, size_t nsy, double thres,
                                                        DevState* st) {
   const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
-  front_range(sx, first, nsx, stride, thres, &st->front[0]);
-  front_range(sy, first, nsy, stride, thres, &st->front[0]);
+  front_range(sx, first, nsx, stride, thres, &st->front[0][0]);
+  front_range(sy, first, nsy, stride, thres, &st->front[0][1]);
 }
 
 __global__ void state_kernel(DevState* st, int op, double t) {
@@ -142,7 +142,7 @@ __global__ void state_kernel(DevState* st, int op, double t) {
     st->frozen_total = 0ull;
     st->bar_count = 0u;
     st->bar_gen = 0u;
-    for (int k = 0; k < 3; ++k) st->front[k] = 0u;
+    for (int k = 0; k < 3; ++k) st->front[k][0] = st->front[k][1] = 0u;
   } else if (op == 2) {  // the barrier's arrivals after a barrier that gave up
     st->bar_count = 0u;
   }

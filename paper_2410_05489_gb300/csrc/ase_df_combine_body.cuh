@@ -109,7 +109,10 @@ __device__ __forceinline__ void combine_range(const GridInfo& g, const CombineAr
     atomicAdd(&a.st->cnt[0], nmarked);
     atomicAdd(&a.st->repaired_total, (unsigned long long)nmarked);
   }
-  if (leader && DIM == 2) a.st->front[a.stage > 0 ? a.stage - 1 : 0] = 0u;  // the stage's sweeps have read it
+  if (leader && DIM == 2) {  // the stage's sweeps have read them
+    unsigned int* front = a.st->front[a.stage > 0 ? a.stage - 1 : 0];
+    front[0] = front[1] = 0u;
+  }
   if (a.stage == 3 && leader) {
     a.st->t += dt;
     a.st->last_dt = dt;
@@ -154,7 +157,10 @@ __device__ __forceinline__ void repair_range(const GridInfo& g, const RepairArgs
       fU = self || (ju >= 0 && marked(i, ju));
     }
     if (!(fL || fR || fD || fU)) continue;
-    if (DIM == 2 && a.front_out != nullptr) *a.front_out = 1u;  // strengths of kSigmaBig
+    if (DIM == 2 && a.front_out != nullptr) {  // strengths of kSigmaBig
+      if (fL || fR) a.front_out[0] = 1u;
+      if (fD || fU) a.front_out[1] = 1u;
+    }
     double F[2][2][C];  // [dir][lower / upper face][component]
 #pragma unroll
     for (int side = 0; side < 2; ++side) {

@@ -104,11 +104,11 @@ struct DevState {
   // Grid barrier of the single-launch repair (repair_all_kernel): arrivals and generation.
   // bar_count is 0 between barriers; ase_df_reset clears both.
   unsigned int bar_count, bar_gen;
-  // front[s]: the strengths that stage s + 1 (or a residual: s = 0) of a 2D problem consumes hold
-  // a front (is_front); raised by the kernel that reads the caller's strengths before the first
-  // stage and by each stage's sweeps and repair for the next, lowered by the consuming stage's
-  // combine.
-  unsigned int front[3];
+  // front[s][d]: the x- (d = 0) or y-face strengths that stage s + 1 (or a residual: s = 0) of a 2D
+  // problem consumes hold a front (is_front); raised by the kernel that reads the caller's strengths
+  // before the first stage and by each stage's sweeps and repair for the next, lowered by the
+  // consuming stage's combine.
+  unsigned int front[3][2];
 };
 
 // Slots of the branch histogram: linear 9th, 7th, 5th order, WENOZ-AO(5,3)+DF, linear 3rd
@@ -143,7 +143,7 @@ struct SweepArgs {
   double* s_out;          // sigma_out of this direction
   DevState* st;
   double tfrac = 0.0;     // the stage's time is st->t + tfrac st->dt (time-dependent ghosts)
-  const unsigned int* front = nullptr;  // whether s_norm, s_tan hold a front (2D; nullptr: no)
+  const unsigned int* front = nullptr;  // [2]: whether the x- and y-face strengths hold a front (2D; nullptr: no)
   unsigned int* front_out = nullptr;    // raised when s_out does (or nullptr)
   unsigned long long* hist = nullptr;  // branch histogram (kBranchSlots counters) or nullptr
 };
@@ -177,7 +177,7 @@ struct RepairArgs {
   int stage;
   int pass;           // 1..kRepairPasses
   double tfrac = 0.0; // the stage's time is st->t + tfrac dt (time-dependent ghosts)
-  unsigned int* front_out = nullptr;  // raised with the strengths of first-order faces (2D)
+  unsigned int* front_out = nullptr;  // [2]: raised with the strengths of first-order faces (2D)
 };
 
 struct SpeedArgs {

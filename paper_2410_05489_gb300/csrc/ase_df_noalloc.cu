@@ -151,7 +151,7 @@ extern "C" ase_df_status ase_df_residual_noalloc(const ase_df_params* pin, const
     a.F = (dir == 0) ? Fx : Fy;
     a.s_out = (dir == 0) ? sx_out : sy_out;
     a.st = st;
-    if (front) a.front = &st->front[0];
+    if (front) a.front = st->front[0];
     switch (p.order) {
       case 3: e = launch_sweep_r3(p.ndim, dir, g, a, *tab, s); break;
       case 5: e = launch_sweep_r5(p.ndim, dir, g, a, *tab, s); break;

@@ -368,13 +368,28 @@ struct TileSpan {
   }
 };
 
+// Whether most of a cell's energy is kinetic (p' = E - |m|^2 / (2 rho) below 2^-9 E) or its values lie
+// beyond 2^+-60: p' then amplifies the rounding of a state by E / p', the strengths of a fast, even
+// stream are that rounding, and the tile keeps to FP64.  From the high words of rho, m, E; in
+// FP32, whose few units in 2^-20 do not matter to the rule.
+__device__ __forceinline__ bool fix_fast(int rho, int mx, int my, int e) {
+  auto f = [](int hi) {  // |x| truncated to 20 bits (0 below 2^-63)
+    const int b = (hi & 0x7fffffff) - (896 << 20);
+    return b < (64 << 20) ? 0.0f : b >= (188 << 20) ? 1e19f : __int_as_float(b << 3);
+  };
+  const float r = f(rho), u = f(mx), v = f(my), en = f(e);
+  return !(r > 0.0f && en > 0.0f && fmaxf(fmaxf(r, en), fmaxf(u, v)) < 1e18f) ||
+         u * u + v * v > 2.0f * (1.0f - 1.0f / 512.0f) * r * en;
+}
+
 // One tile: faces a0 .. a0+TN-1 along the sweep on lines b0 .. b0+tt-1, 1 <= tt <= TT
 // (threadIdx.x is the worker index); smem holds Tile<R, DIM, TT>::sweep_doubles doubles,
 // laid out for TT lines whatever tt is.
 //
-// 2D flows with a front (some face strength of the problem is beyond smooth_limit, below which
-// every branch is linear) take both reconstructions in fixed point on the integer units
-// (ase_df_fixed.cuh) in the tiles whose density and energy span few binades (TileSpan::fits),
+// 2D flows with a front in both directions (some x-face and some y-face strength beyond smooth_limit,
+// below which every branch is linear) take both reconstructions in fixed point on the integer units
+// (ase_df_fixed.cuh) in the tiles whose density and energy span few binades (TileSpan::fits,
+// fix_fast),
 // wherever the branch is the linear one of order R; the FP64 pipe is left to the Gauss points.
 // The other branches run in FP64 in second passes over queues of such cells and faces.  Normal
 // values are then kept in shared memory as limbs at the tile's exponents.  An order-9 face then
@@ -383,9 +398,10 @@ struct TileSpan {
 // the 1600 x 800 order-9 jet residual 3700 -> 2653 us; 64 mixed problems 14.5 -> 11.1 ms.  Exponents
 // per line with aligned sums measured 1046 / 2708 us / 13.0 ms: the alignment costs instructions,
 // and lines crossing a strong front made their tiles slower than plain FP64.
-// Flows without a front stay in FP64 to the bit: their strengths are differences of two
+// Flows without a front in both directions stay in FP64 to the bit: their strengths are differences of two
 // reconstructions that agree to rounding (1e-12 made of 1e-16 parts on a fine smooth grid), so
-// any other rounding of a state, however exact, shows in the fifth digit of the strengths.
+// any other rounding of a state, however exact, shows in the fifth digit of the strengths; with a
+// front across one direction only (a wall, a tube), the other direction's strengths are such.
 template <int R, int DIM, int DIR, int TT_ = (DIM == 2) ? 64 : 1, int TN_ = (DIM == 2) ? 8 : 255, int NT_ = 256>
 __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& args, const Tables& T, int a0,
                                            int b0, int tt, double* smem) {
@@ -432,7 +448,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   if (DIM == 2 && tid == 0) *s_any = 0;
   Limbs* iQP = reinterpret_cast<Limbs*>(sQP);
   Limbs* iQM = reinterpret_cast<Limbs*>(sQM);
-  const bool front = DIM == 2 && args.front != nullptr && *args.front != 0u;
+  const bool front = DIM == 2 && args.front != nullptr && args.front[0] != 0u && args.front[1] != 0u;
   const unsigned long long limit = smooth_limit(g.thres);
   // ---- staging: consecutive threads take consecutive addresses along the direction in which the
   // arrays are contiguous (the sweep for x-faces, the lines for y-faces) ----
@@ -471,6 +487,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       }
     }
   }
+  bool fast = false;  // a staged cell that asks for FP64 (fix_fast)
   if (front) {
     if constexpr (DIM == 2 && TT == 32) {
       // a tile of 32 lines takes the exponents of the 64-line tile it is half of, so that the tile
@@ -478,9 +495,14 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       const int bx = (b0 & 32) ? b0 - 32 - KT : b0 + 32 + KT;
       for (int idx = tid; idx < 32 * NA; idx += NT) {
         const int a = a0 - 1 - K + ((DIR == 0) ? idx % NA : idx / 32), b = bx + ((DIR == 0) ? idx / NA : idx % 32);
-#pragma unroll 1
-        for (int c = 0; c < C; ++c)
-          span.add(c, C - 1, (DIR == 0) ? fetch_w(g, args.W, c, a, b, ts) : fetch_w(g, args.W, c, b, a, ts));
+        int hi[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          const double v = (DIR == 0) ? fetch_w(g, args.W, c, a, b, ts) : fetch_w(g, args.W, c, b, a, ts);
+          span.add(c, C - 1, v);
+          hi[c] = (int)(dbits(v) >> 32);
+        }
+        fast |= fix_fast(hi[0], hi[1], hi[2], hi[3]);
       }
     }
     span.store(s_part);
@@ -526,7 +548,12 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   int ex[3];  // exponents of density, momentum, energy
   if (front) {
     span.load(s_part, NT / 32);
-    fixed = span.fits();
+    if constexpr (DIM == 2) {
+      const int* hi = reinterpret_cast<const int*>(sW) + 1;
+      for (int idx = tid; idx < nb * NA; idx += NT)
+        fast |= fix_fast(hi[2 * idx], hi[2 * (NB * NA + idx)], hi[2 * (2 * NB * NA + idx)], hi[2 * (3 * NB * NA + idx)]);
+    }
+    fixed = !__syncthreads_or(fast) && span.fits();
     ex[0] = fix_exponent(exp_of(span.rmax));
     ex[1] = fix_exponent(exp_of(span.mmax));
     ex[2] = fix_exponent(exp_of(span.emax));
