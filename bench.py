@@ -41,7 +41,7 @@ HBM_BYTES_PER_CELL_STAGE_2D = 128.0  # read W^(s), W^n, write W^(s+1), sigma in/
 # Sources of the face-sweep kernel: the ncu summaries under profiles/ record a hash of these
 # files beside their counters, and the counters are reported only while the hash matches.
 SWEEP_SOURCES = ("ase_df_sweep.cu", "ase_df_sweep_body.cuh", "ase_df_device.cuh", "ase_df_internal.cuh",
-                 "ase_df_tileplan.h")
+                 "ase_df_tileplan.h", "ase_df_fixed.cuh", "ase_df_imul.cuh")
 SWEEP_PROFILE = {9: "sweep_kernel_r9_2d_vortex1024_ncu.md", 7: "sweep_kernel_r7_2d_vortex1024_ncu.md"}
 
 
