@@ -394,7 +394,8 @@ __device__ __forceinline__ bool fix_fast(int rho, int mx, int my, int e) {
 // The other branches run in FP64 in second passes over queues of such cells and faces.  Normal
 // values are then kept in shared memory as limbs at the tile's exponents.  An order-9 face then
 // takes 287 FP64 instructions instead of 586 (pipe 72 % busy, the rest waits on the 16 resident
-// warps).  Measured, FP64 -> fixed point: Configuration 3 512^2 order 5, one step, 1350 -> 1013 us;
+// warps); 187 since the products of the Gauss points left the pipe as well (ase_df_imul.cuh).  Measured
+// before that, FP64 -> fixed point: Configuration 3 512^2 order 5, one step, 1350 -> 1013 us;
 // the 1600 x 800 order-9 jet residual 3700 -> 2653 us; 64 mixed problems 14.5 -> 11.1 ms.  Exponents
 // per line with aligned sums measured 1046 / 2708 us / 13.0 ms: the alignment costs instructions,
 // and lines crossing a strong front made their tiles slower than plain FP64.
