@@ -352,11 +352,11 @@ const char* ase_df_last_error(const ase_df_ctx* c) { return c ? c->err : g_init_
 // launch sequences
 // ---------------------------------------------------------------------------------
 static cudaError_t sweep(ase_df_ctx* c, int dir, const double* W, const double* sx, const double* sy,
-                         double* F, double* s_out, cudaStream_t s, double tfrac, int stage) {
+                         double* F, double* s_out, cudaStream_t s, double tfrac, int stage, bool next) {
   SweepArgs a;
   if (stage >= 0 && looks_for_front(c->dim, c->g, c->p.order)) {
     a.front = c->st->front[stage > 0 ? stage - 1 : 0];
-    if (stage == 1 || stage == 2) a.front_out = &c->st->front[stage][dir];
+    if (next) a.front_out = &c->st->front[stage][dir];
   }
   a.tfrac = tfrac;
   a.W = W;
@@ -383,19 +383,21 @@ static cudaError_t sweep(ase_df_ctx* c, int dir, const double* W, const double* 
 // so that each launch is timed alone.
 // stage: 0 a residual, 1..3 the SSP-RK3 stages, -1 priming (zero strengths: no front).  A
 // residual's and a first stage's front[0] has been set before (launch_strength, or the CFL
-// kernel); stages 1 and 2 raise the next stage's.
+// kernel).  next: the call's next stage consumes the strengths that this one leaves, and finds
+// front[stage] raised when they hold a front.  Only that stage's combine lowers it again, so
+// a call whose last sweep is this one must not raise it: a later call would read it.
 static cudaError_t face_fluxes(ase_df_ctx* c, const double* W, const double* sx, const double* sy,
-                               double* sxo, double* syo, cudaStream_t s, int stage, double tfrac = 0.0) {
+                               double* sxo, double* syo, cudaStream_t s, int stage, bool next, double tfrac = 0.0) {
   if (c->dim == 1 || c->prof_on) {
-    cudaError_t e = sweep(c, 0, W, sx, sy, c->Fx, sxo, s, tfrac, stage);
+    cudaError_t e = sweep(c, 0, W, sx, sy, c->Fx, sxo, s, tfrac, stage, next);
     if (e != cudaSuccess || c->dim == 1) return e;
-    return sweep(c, 1, W, sx, sy, c->Fy, syo, s, tfrac, stage);
+    return sweep(c, 1, W, sx, sy, c->Fy, syo, s, tfrac, stage, next);
   }
   cudaError_t e = cudaEventRecord(c->ev_fork, s);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side, c->ev_fork, 0);
   if (e != cudaSuccess) return e;
-  cudaError_t ex = sweep(c, 0, W, sx, sy, c->Fx, sxo, s, tfrac, stage);
-  cudaError_t ey = sweep(c, 1, W, sx, sy, c->Fy, syo, c->side, tfrac, stage);
+  cudaError_t ex = sweep(c, 0, W, sx, sy, c->Fx, sxo, s, tfrac, stage, next);
+  cudaError_t ey = sweep(c, 1, W, sx, sy, c->Fy, syo, c->side, tfrac, stage, next);
   // the join is made whatever happened, so that s never runs ahead of the side stream
   e = cudaEventRecord(c->ev_join, c->side);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->ev_join, 0);
@@ -407,9 +409,9 @@ static cudaError_t face_fluxes(ase_df_ctx* c, const double* W, const double* sx,
 static double rk_tfrac(int stage) { return stage == 2 ? 1.0 : (stage == 3 ? 0.5 : 0.0); }
 
 // Stage combination (or L for stage 0); for stages 1..3 followed by the positivity
-// repair passes, which get the stage's sigma_out (sxo, syo).
+// repair passes, which get the stage's sigma_out (sxo, syo); next as in face_fluxes.
 static cudaError_t combine(ase_df_ctx* c, int stage, const double* Wn, const double* Ws, double* out,
-                           double dt_fixed, cudaStream_t s, double* sxo = nullptr, double* syo = nullptr) {
+                           double dt_fixed, cudaStream_t s, bool next, double* sxo = nullptr, double* syo = nullptr) {
   cudaError_t e = cudaSuccess;
   CombineArgs a;
   a.mark = c->mark;
@@ -448,7 +450,7 @@ static cudaError_t combine(ase_df_ctx* c, int stage, const double* Wn, const dou
   r.dt_fixed = dt_fixed;
   r.stage = stage;
   r.tfrac = rk_tfrac(stage);
-  if (stage < 3 && looks_for_front(c->dim, c->g, c->p.order)) r.front_out = c->st->front[stage];
+  if (next && looks_for_front(c->dim, c->g, c->p.order)) r.front_out = c->st->front[stage];
   r.pass = 1;
   if (small) return launch_combine_repair(c->g, a, r, s);
   ProfScope prof(c, s, 4);
@@ -485,14 +487,14 @@ static ase_df_status step_launches(ase_df_ctx* c, double* W, double* sx, double*
   }
   const double dtf = (dt > 0.0) ? dt : 0.0;
   // stage 1
-  if ((e = face_fluxes(c, W, sx, sy, c->sxa, c->sya, s, 1)) != cudaSuccess) return cuda_fail(c, e, "stage 1 sweep");
-  if ((e = combine(c, 1, W, W, c->W1, dtf, s, c->sxa, c->sya)) != cudaSuccess) return cuda_fail(c, e, "stage 1 combine");
+  if ((e = face_fluxes(c, W, sx, sy, c->sxa, c->sya, s, 1, true)) != cudaSuccess) return cuda_fail(c, e, "stage 1 sweep");
+  if ((e = combine(c, 1, W, W, c->W1, dtf, s, true, c->sxa, c->sya)) != cudaSuccess) return cuda_fail(c, e, "stage 1 combine");
   // stage 2
-  if ((e = face_fluxes(c, c->W1, c->sxa, c->sya, c->sxb, c->syb, s, 2, rk_tfrac(2))) != cudaSuccess) return cuda_fail(c, e, "stage 2 sweep");
-  if ((e = combine(c, 2, W, c->W1, c->W2, dtf, s, c->sxb, c->syb)) != cudaSuccess) return cuda_fail(c, e, "stage 2 combine");
+  if ((e = face_fluxes(c, c->W1, c->sxa, c->sya, c->sxb, c->syb, s, 2, true, rk_tfrac(2))) != cudaSuccess) return cuda_fail(c, e, "stage 2 sweep");
+  if ((e = combine(c, 2, W, c->W1, c->W2, dtf, s, true, c->sxb, c->syb)) != cudaSuccess) return cuda_fail(c, e, "stage 2 combine");
   // stage 3: sigma_out lands in the caller's sx / sy, W^{n+1} in W
-  if ((e = face_fluxes(c, c->W2, c->sxb, c->syb, sx, sy, s, 3, rk_tfrac(3))) != cudaSuccess) return cuda_fail(c, e, "stage 3 sweep");
-  if ((e = combine(c, 3, W, c->W2, W, dtf, s, sx, sy)) != cudaSuccess) return cuda_fail(c, e, "stage 3 combine");
+  if ((e = face_fluxes(c, c->W2, c->sxb, c->syb, sx, sy, s, 3, false, rk_tfrac(3))) != cudaSuccess) return cuda_fail(c, e, "stage 3 sweep");
+  if ((e = combine(c, 3, W, c->W2, W, dtf, s, false, sx, sy)) != cudaSuccess) return cuda_fail(c, e, "stage 3 combine");
   return ASE_DF_OK;
 }
 
@@ -508,9 +510,9 @@ ase_df_status ase_df_residual(ase_df_ctx* c, const double* W, const double* sx_i
   cudaStream_t s = (cudaStream_t)stream;
   c->last_stream = s;
   cudaError_t e = looks_for_front(c->dim, c->g, c->p.order) ? launch_strength(c->g, sx_in, sy_in, c->st, s) : cudaSuccess;
-  if (e == cudaSuccess) e = face_fluxes(c, W, sx_in, sy_in, sx_out, sy_out, s, 0);
+  if (e == cudaSuccess) e = face_fluxes(c, W, sx_in, sy_in, sx_out, sy_out, s, 0, false);
   if (e != cudaSuccess) return cuda_fail(c, e, "residual sweep");
-  e = combine(c, 0, W, W, L, 0.0, s);
+  e = combine(c, 0, W, W, L, 0.0, s, false);
   if (e != cudaSuccess) return cuda_fail(c, e, "residual combine");
   return ASE_DF_OK;
 }
@@ -520,7 +522,7 @@ ase_df_status ase_df_prime_sigma(ase_df_ctx* c, const double* W, double* sx, dou
   if (r != ASE_DF_OK) return r;
   cudaStream_t s = (cudaStream_t)stream;
   c->last_stream = s;
-  cudaError_t e = face_fluxes(c, W, c->zsx, c->zsy, sx, sy, s, -1);
+  cudaError_t e = face_fluxes(c, W, c->zsx, c->zsy, sx, sy, s, -1, false);
   if (e != cudaSuccess) return cuda_fail(c, e, "prime_sigma");
   return ASE_DF_OK;
 }
@@ -745,10 +747,10 @@ ase_df_status ase_df_step_adjoint(ase_df_ctx* c, const double* W, const double* 
   // stages 1 and 2 of the forward step: W1, sigma1 (sxa, sya), W2, sigma2 (sxb, syb)
   if (looks_for_front(c->dim, c->g, c->p.order) && (e = launch_strength(c->g, sx, sy, c->st, s)) != cudaSuccess)
     return cuda_fail(c, e, "adjoint: strength scan");
-  if ((e = face_fluxes(c, W, sx, sy, c->sxa, c->sya, s, 1)) != cudaSuccess) return cuda_fail(c, e, "adjoint: stage 1 sweep");
-  if ((e = combine(c, 1, W, W, c->W1, dt, s, c->sxa, c->sya)) != cudaSuccess) return cuda_fail(c, e, "adjoint: stage 1 combine");
-  if ((e = face_fluxes(c, c->W1, c->sxa, c->sya, c->sxb, c->syb, s, 2, rk_tfrac(2))) != cudaSuccess) return cuda_fail(c, e, "adjoint: stage 2 sweep");
-  if ((e = combine(c, 2, W, c->W1, c->W2, dt, s, c->sxb, c->syb)) != cudaSuccess) return cuda_fail(c, e, "adjoint: stage 2 combine");
+  if ((e = face_fluxes(c, W, sx, sy, c->sxa, c->sya, s, 1, true)) != cudaSuccess) return cuda_fail(c, e, "adjoint: stage 1 sweep");
+  if ((e = combine(c, 1, W, W, c->W1, dt, s, true, c->sxa, c->sya)) != cudaSuccess) return cuda_fail(c, e, "adjoint: stage 1 combine");
+  if ((e = face_fluxes(c, c->W1, c->sxa, c->sya, c->sxb, c->syb, s, 2, false, rk_tfrac(2))) != cudaSuccess) return cuda_fail(c, e, "adjoint: stage 2 sweep");
+  if ((e = combine(c, 2, W, c->W1, c->W2, dt, s, false, c->sxb, c->syb)) != cudaSuccess) return cuda_fail(c, e, "adjoint: stage 2 combine");
   // stage 3: W^{n+1} = W^n / 3 + 2/3 W2 + 2/3 dt L(W2, sigma2), sigma3 = sigma_out(W2, sigma2)
   e = launch_axpby(c->Abn, 1.0 / 3.0, Wbar, 0.0, nullptr, nW, s);
   if (e == cudaSuccess) e = launch_axpby(c->Ab2, 2.0 / 3.0, Wbar, 0.0, nullptr, nW, s);
