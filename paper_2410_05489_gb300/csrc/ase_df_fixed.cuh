@@ -6,33 +6,37 @@
 // weights, so they can leave the FP64 pipe to the Gauss-point flux: the 1024^2 order-9 sweep
 // spent 321 of its 586 FP64 instructions per face on them.
 //
-// The values of a component in a tile share one exponent e (the largest of theirs):
-//   v = M 2^(e - 1023 - 56), |M| < 2^57,
-// so M keeps 4 bits below the last bit of a double of exponent e.  Weights are integers in
-// units of 2^-56 that sum to 2^56 exactly (constant data are reproduced), split like M into
-// limbs of 28 bits, w = wh 2^28 + wl with |wl| <= 2^27.  With M = mh 2^28 + ml,
-//   sum w M / 2^56 = sum mh wh + (sum mh wl + ml wh) / 2^28 + (sum ml wl) / 2^56,
+// The values of ONE stencil share one exponent e, that of the largest:
+//   |v| = M 2^(e - 1023 - 56), M < 2^57.
+// A stencil whose values have one sign and lie within kFixRange binades is exact in M, so the result
+// is a function of the stencil's values alone, whichever tile or launch evaluates it, and an error
+// is relative to these values.  (A momentum that changes sign in the stencil, or a value far below its
+// neighbours, takes the FP64 chain; zeros throughout give zero.)
+// Weights are integers in units of 2^-56 that sum to 2^56 exactly.  The sum is therefore formed as
+//   M_0 + sum w_t (M_t - M_0) / 2^56
+// which reproduces constant data to the bit.  With differences and weights in limbs of 28 bits,
+// d = dh 2^28 + dl and w = wh 2^28 + wl, |wl| <= 2^27,
+//   sum w d / 2^56 = sum dh wh + (sum dh wl + dl wh) / 2^28 + (sum dl wl) / 2^56,
 // and the last sum, below half a unit of M per term, is left out: three multiply-adds per
-// term into two 64-bit sums, with an error of about a unit, 2^-56 of the tile's largest value
-// (a chain of nine FP64 multiply-adds makes up to 2^-51 of it).
-// Bounds: |value| <= 1.79 |M| for one reconstruction (the weights' absolute sum at order 9), so a
-// normal reconstruction stays below 2^57.9, its tangential sums S = W_t + W_-t below 2^58.9
-// (their high limb below 2^31), and the two 64-bit sums below 2^62.
+// term into two 64-bit sums and one rounding to double.  Measured against exact sums over stencils that span
+// 0 to kFixRange binades (host test), the rms error is 0.4 to 0.7 of the FP64 chain's.
+// Bounds: |M_t - M_0| < 2^57, so its high limb is below 2^29, that of (M_t - M_0) + (M_-t - M_0) below
+// 2^30; the weights' absolute sum without the centre's is below 1.1, so results stay below 2^59
+// and both 64-bit sums below 2^61.
 #pragma once
 
-#include "ase_df_device.cuh"
+#include <cuda_runtime.h>
 
 namespace asedf {
 namespace {
 
-constexpr int kFixBits = 56;  // fraction bits of M at the shared exponent, and of the weights
+constexpr int kFixBits = 56;  // fraction bits of M at the stencil's exponent, and of the weights
 constexpr int kLimb = 28;
-// Tiles with a larger biased exponent (values above 2^240) take the FP64 path, whose nonlinear
-// weights overflow there.
-constexpr int kFixMaxExp = 1023 + 240;
-// The shared exponents serve a tile whose density and energy stay within this many binades: the
-// smallest value then still has 52 bits above the unit of M.
-constexpr int kFixRange = 4;
+// Biased exponents of a stencil's largest value: not below 64 (results stay normal) nor beyond 2^240
+// (infinities and NaN, and values whose nonlinear weights overflow elsewhere).
+constexpr int kFixMinExp = 64, kFixMaxExp = 1023 + 240;
+// Largest difference between the exponents of a stencil.
+constexpr int kFixRange = 3;
 
 // Weights of the order-r linear branch (index (r - 3) / 2), high and low limbs:
 //   f: W_t, t = -k..k, at xi = 0 (xi = -1 is its mirror image);
@@ -75,58 +79,134 @@ struct Limbs {
   int h, l;
 };
 
-__device__ __forceinline__ Limbs fix_split(long long m) {
-  return Limbs{(int)(m >> kLimb), (int)m & ((1 << kLimb) - 1)};
+// M of the magnitude of a normal double; k = 8 - (e - its exponent), 4 < k <= 8.
+__device__ __forceinline__ Limbs fix_from_double(int hi, int lo, int k) {
+  const unsigned a = (unsigned)((hi & 0xfffff) | 0x100000);
+  return Limbs{(int)__funnelshift_l((unsigned)lo, a, k), (int)(((unsigned)lo << k) >> 4)};
 }
 
-// Two-limb sum of products; the rounding half of the final shift is the starting value.
+// Two-limb sum, in units of 1 and 2^-28.
 struct FixSum {
   long long hh, mid;
 };
-__device__ __forceinline__ FixSum fix_zero() { return FixSum{0ll, 1ll << (kLimb - 1)}; }
-__device__ __forceinline__ void fix_mad(FixSum& s, Limbs m, int wh, int wl) {
-  s.hh += (long long)m.h * wh;
-  s.mid += (long long)m.h * wl;
-  s.mid += (long long)m.l * wh;
-}
-__device__ __forceinline__ long long fix_value(FixSum s) { return s.hh + (s.mid >> kLimb); }
-
-// Biased exponent of |x| from its high word (sign cleared).
-__device__ __forceinline__ int exp_of(int abs_hi) { return (int)((unsigned)abs_hi >> 20); }
-
-// The exponent values of largest biased exponent emax are kept at: not below 64, so that zeros
-// and subnormals (far more than 57 binades below) become 0.
-__device__ __forceinline__ int fix_exponent(int emax) { return emax < 64 ? 64 : emax; }
-
-// M of a finite double at shared exponent e (biased exponent of x at most e + 1): the 53-bit
-// significand shifted into place, truncated toward zero, sign applied to both limbs.
-__device__ __forceinline__ Limbs fix_from_double(double x, int e) {
-  const long long b = dbits(x);
-  const int hi = (int)(b >> 32);
-  int d = e + 1 - ((hi >> 20) & 0x7ff);
-  d = d > 63 ? 63 : d;
-  const unsigned long long sig =
-      ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)b) << (kFixBits - 51);
-  const unsigned long long m = sig >> d;
-  const int s = hi >> 31;
-  const int h = (int)(m >> kLimb), l = (int)m & ((1 << kLimb) - 1);
-  return Limbs{(h ^ s) - s, (l ^ s) - s};
+__device__ __forceinline__ void fix_mad(FixSum& s, Limbs d, int wh, int wl) {
+  s.hh += (long long)d.h * wh;
+  s.mid += (long long)d.h * wl;
+  s.mid += (long long)d.l * wh;
 }
 
-__device__ __forceinline__ long long fix_join(Limbs m) { return ((long long)m.h << kLimb) + m.l; }
-
-// The double nearest to R 2^(e - 1023 - 56), |R| < 2^62, 64 <= e <= 2046 - 62 (ties away from zero).
-__device__ __forceinline__ double fix_to_double(long long R, int e) {
-  const long long s = R >> 63;
-  const unsigned long long a = (unsigned long long)((R ^ s) - s);
+// The double nearest to +- s 2^(e - 1023 - 56), |s| < 2^61, kFixMinExp <= e <= kFixMaxExp; sign: 0, or
+// the sign bit of the stencil's values.
+__device__ __forceinline__ double fix_to_double(FixSum s, int e, unsigned sign) {
+  const long long R = s.hh + ((s.mid + (1ll << (kLimb - 1))) >> kLimb), n = R >> 63;
+  const unsigned long long a = (unsigned long long)((R ^ n) - n);
   // leading bit from a truncating conversion of the upper (or only) non-zero word
   const unsigned ah = (unsigned)(a >> 32);
   const unsigned w = ah != 0u ? ah : (unsigned)a;
   const int lead = (__float_as_int(__uint2float_rz(w)) >> 23) - (ah != 0u ? 95 : 127);  // for a != 0
   const unsigned long long m = ((a << ((62 - lead) & 63)) + 0x200u) >> 10;  // 53 bits, or 2^53
   const unsigned hi = (unsigned)(m >> 32) + ((unsigned)(e + lead - kFixBits - 1) << 20);
-  const unsigned long long bits = (unsigned long long)(hi | ((unsigned)s & 0x80000000u)) << 32 | (unsigned)m;
+  const unsigned long long bits = (unsigned long long)(hi | (((unsigned)n & 0x80000000u) ^ sign)) << 32 | (unsigned)m;
   return __longlong_as_double(a == 0ull ? 0ll : (long long)bits);
+}
+
+// A stencil of 2 K + 1 values in fixed point.
+template <int K>
+struct FixStencil {
+  int e;
+  unsigned sign;     // sign bit of the values
+  long long m0;      // the centre
+  Limbs p[K], m[K];  // W_t - W_0 and W_-t - W_0, t = 1 .. K
+
+  // v points at W_0, W_t at v[t vs].  Returns 1; 0 when the stencil does not fit; -1 when it is all zeros.
+  __device__ __forceinline__ int load(const double* v, int vs) {
+    int hi[2 * K + 1], lo[2 * K + 1];
+    int mx = -0x7fffffff, mn = 0x7fffffff;  // of the exponents, less 2048 for negative values
+#pragma unroll
+    for (int t = 0; t <= 2 * K; ++t) {
+      const long long b = __double_as_longlong(v[(t - K) * vs]);
+      hi[t] = (int)(b >> 32);
+      lo[t] = (int)b;
+      mx = max(mx, hi[t] >> 20);
+      mn = min(mn, hi[t] >> 20);
+    }
+    e = mx & 0x7ff;
+    sign = (unsigned)mx & 0x80000000u;
+    if (mx - mn > kFixRange || (unsigned)(e - kFixMinExp) > (unsigned)(kFixMaxExp - kFixMinExp)) {
+      int any = 0;
+#pragma unroll
+      for (int t = 0; t <= 2 * K; ++t) any |= (hi[t] & 0x7fffffff) | lo[t];
+      return any == 0 ? -1 : 0;
+    }
+    const Limbs c = fix_from_double(hi[K], lo[K], (hi[K] >> 20) - mx + 8);
+    m0 = (long long)c.h * (1 << kLimb) + c.l;
+#pragma unroll
+    for (int t = 1; t <= K; ++t) {
+      const Limbs a = fix_from_double(hi[K + t], lo[K + t], (hi[K + t] >> 20) - mx + 8);
+      const Limbs b = fix_from_double(hi[K - t], lo[K - t], (hi[K - t] >> 20) - mx + 8);
+      p[t - 1] = Limbs{a.h - c.h, a.l - c.l};
+      m[t - 1] = Limbs{b.h - c.h, b.l - c.l};
+    }
+    return 1;
+  }
+};
+
+// Order-R linear reconstruction at the upper face (xi = 0) of the stencil's cell and, with NP = 2,
+// at the lower one (xi = -1: the mirrored weights).  Returns whether the stencil fits.
+template <int R, int NP>
+__device__ __forceinline__ bool fix_normal(const double* v, int vs, double* out) {
+  constexpr int K = (R - 1) / 2;
+  const FixWeights& F = kFixW[(R - 3) / 2];
+  FixStencil<K> s;
+  const int fit = s.load(v, vs);
+  if (fit <= 0) {
+#pragma unroll
+    for (int q = 0; q < NP; ++q) out[q] = 0.0;
+    return fit != 0;
+  }
+#pragma unroll
+  for (int q = 0; q < NP; ++q) {
+    FixSum x{s.m0, 0ll};
+#pragma unroll
+    for (int t = 1; t <= K; ++t) {
+      fix_mad(x, q == 0 ? s.p[t - 1] : s.m[t - 1], F.fh[K + t], F.fl[K + t]);
+      fix_mad(x, q == 0 ? s.m[t - 1] : s.p[t - 1], F.fh[K - t], F.fl[K - t]);
+    }
+    out[q] = fix_to_double(x, s.e, s.sign);
+  }
+  return true;
+}
+
+// Gauss-point values of the order-R linear branch by the even and odd sums of lin_gauss_sym: the
+// points eta and -1 - eta are E +- O.  Returns whether the stencil fits.
+template <int R, int G>
+__device__ __forceinline__ bool fix_gauss(const double* v, int vs, double* out) {
+  constexpr int K = (R - 1) / 2;
+  const FixWeights& F = kFixW[(R - 3) / 2];
+  FixStencil<K> s;
+  const int fit = s.load(v, vs);
+  if (fit <= 0) {
+#pragma unroll
+    for (int q = 0; q < G; ++q) out[q] = 0.0;
+    return fit != 0;
+  }
+#pragma unroll
+  for (int g = 0; g < (G + 1) / 2; ++g) {
+    FixSum E{s.m0, 0ll}, O{0ll, 0ll};
+#pragma unroll
+    for (int t = 1; t <= K; ++t)
+      fix_mad(E, Limbs{s.p[t - 1].h + s.m[t - 1].h, s.p[t - 1].l + s.m[t - 1].l}, F.eh[g][t], F.el[g][t]);
+    if (2 * g + 1 == G) {
+      out[g] = fix_to_double(E, s.e, s.sign);  // middle point
+    } else {
+#pragma unroll
+      for (int t = 1; t <= K; ++t)
+        fix_mad(O, Limbs{s.p[t - 1].h - s.m[t - 1].h, s.p[t - 1].l - s.m[t - 1].l}, F.oh[g][t], F.ol[g][t]);
+      out[g] = fix_to_double(FixSum{E.hh + O.hh, E.mid + O.mid}, s.e, s.sign);
+      out[G - 1 - g] = fix_to_double(FixSum{E.hh - O.hh, E.mid - O.mid}, s.e, s.sign);
+    }
+  }
+  return true;
 }
 
 }  // namespace

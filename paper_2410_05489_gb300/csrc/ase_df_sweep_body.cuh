@@ -36,13 +36,11 @@ __device__ __forceinline__ Branch select_branch(const double* s, double thres) {
   // thres/16 (compared as unsigned bit patterns, so negative values and NaN fail), each
   // stencil sum is at most 8 thres/16 = thres/2 also after rounding (rounded addition is
   // monotone in its operands), so every sum is below thres and the branch is linear order R.
-  {
-    const unsigned long long lim = smooth_limit(thres);
-    unsigned long long mx = (unsigned long long)dbits(s[0]);
+  const unsigned long long lim = smooth_limit(thres);
+  unsigned long long mx = (unsigned long long)dbits(s[0]);
 #pragma unroll
-    for (int t = 1; t < 2 * K; ++t) mx = max(mx, (unsigned long long)dbits(s[t]));
-    if (mx <= lim) return b;
-  }
+  for (int t = 1; t < 2 * K; ++t) mx = max(mx, (unsigned long long)dbits(s[t]));
+  if (mx <= lim) return b;
   const double sm12 = s[K - 1], sp12 = s[K];  // sigma_{-1/2}, sigma_{1/2}
   if (R == 3) {
     const double A = sm12 + sp12;
@@ -230,9 +228,9 @@ struct Tile {
   static constexpr size_t queue_offset =
       (size_t)C * NB * NA + 2 * (size_t)C * NB * NQ + (size_t)NB * NSN + (DIM == 2 ? (size_t)NQ * NST : 0);
   static constexpr size_t smem_doubles = queue_offset + ((size_t)QCAP + 2 + 1) / 2;
-  // 2D sweeps, after the queue: a flag (2 ints) and 8 ints per warp (TileSpan)
-  static constexpr size_t span_offset = smem_doubles;
-  static constexpr size_t split_offset = smem_doubles + (DIM == 2 ? 1 + (size_t)(NT / 32) * 4 : 0);
+  // 2D sweeps, after the queue: a word of fast cells per staged line and per line of faces (fix_fast)
+  static constexpr size_t fast_offset = smem_doubles;
+  static constexpr size_t split_offset = smem_doubles + (DIM == 2 ? ((size_t)NB + TT + 1) / 2 : 0);
   // 2D tiles of 16 lines, last: the states [2][G][C] and terms [5][G] of every face and the
   // branches (5 words) of its columns (sweep_tile)
   static constexpr bool split = DIM == 2 && TT == 16;
@@ -273,105 +271,10 @@ __device__ __forceinline__ bool defer_item(bool defer, int item, int* queue, uns
   return defer;
 }
 
-// One component of one staged line in fixed point at the tile's exponent e: the order-R linear
-// reconstruction of its NQ cells at both faces (the two end cells at one).  The line's cell
-// averages are converted once and serve all of its stencils.
-template <int R, int NA, int NQ>
-__device__ __forceinline__ void fix_line(const double* v, int e, Limbs* qp, Limbs* qm) {
-  constexpr int K = (R - 1) / 2;
-  const FixWeights& F = kFixW[(R - 3) / 2];
-  Limbs m[NA];
-#pragma unroll
-  for (int t = 0; t < NA; ++t) m[t] = fix_from_double(v[t], e);
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    if (q < NQ - 1) {
-      FixSum s = fix_zero();
-#pragma unroll
-      for (int t = 0; t <= 2 * K; ++t) fix_mad(s, m[q + t], F.fh[t], F.fl[t]);
-      qp[q] = fix_split(fix_value(s));
-    }
-    if (q > 0) {
-      FixSum s = fix_zero();
-#pragma unroll
-      for (int t = 0; t <= 2 * K; ++t) fix_mad(s, m[q + t], F.fh[2 * K - t], F.fl[2 * K - t]);
-      qm[q] = fix_split(fix_value(s));
-    }
-  }
-}
-
-// Gauss-point values of the order-R linear branch from the normal values Q (stride NQ) of lines
-// -K .. K: the even and odd sums of lin_gauss_sym in fixed point.  The limbs add without carry.
-template <int R, int G, int NQ>
-__device__ __forceinline__ void fix_gauss(const Limbs* Q, int e, double* out) {
-  constexpr int K = (R - 1) / 2;
-  const FixWeights& F = kFixW[(R - 3) / 2];
-  Limbs S[K + 1], D[K + 1];
-  S[0] = Q[0];
-#pragma unroll
-  for (int t = 1; t <= K; ++t) {
-    const Limbs a = Q[t * NQ], b = Q[-t * NQ];
-    S[t] = Limbs{a.h + b.h, a.l + b.l};
-    D[t] = Limbs{a.h - b.h, a.l - b.l};
-  }
-#pragma unroll
-  for (int g = 0; g < (G + 1) / 2; ++g) {
-    FixSum E = fix_zero();
-#pragma unroll
-    for (int t = 0; t <= K; ++t) fix_mad(E, S[t], F.eh[g][t], F.el[g][t]);
-    const long long ev = fix_value(E);
-    if (2 * g + 1 == G) {
-      out[g] = fix_to_double(ev, e);  // middle point
-    } else {
-      FixSum O = fix_zero();
-#pragma unroll
-      for (int t = 1; t <= K; ++t) fix_mad(O, D[t], F.oh[g][t], F.ol[g][t]);
-      const long long ov = fix_value(O);
-      out[g] = fix_to_double(ev + ov, e);
-      out[G - 1 - g] = fix_to_double(ev - ov, e);
-    }
-  }
-}
-
-// What a tile's staged cell averages span, on the high words of the doubles: largest and smallest
-// of density and energy, largest momentum magnitude (each thread its own, then the CTA's).
-struct TileSpan {
-  int rmax = 0, rmin = 0x7fffffff, emax = 0, emin = 0x7fffffff, mmax = 0;
-  __device__ __forceinline__ void add(int c, int last, double v) {
-    const int hi = (int)(dbits(v) >> 32);
-    if (c == 0) { rmax = max(rmax, hi & 0x7fffffff); rmin = min(rmin, hi); }
-    else if (c == last) { emax = max(emax, hi & 0x7fffffff); emin = min(emin, hi); }
-    else mmax = max(mmax, hi & 0x7fffffff);
-  }
-  // s_part: 8 ints per warp; store before and load after a barrier
-  __device__ __forceinline__ void store(int* s_part) const {
-    const int v[5] = {__reduce_max_sync(0xffffffffu, rmax), __reduce_min_sync(0xffffffffu, rmin),
-                      __reduce_max_sync(0xffffffffu, emax), __reduce_min_sync(0xffffffffu, emin),
-                      __reduce_max_sync(0xffffffffu, mmax)};
-    if ((threadIdx.x & 31) == 0)
-      for (int k = 0; k < 5; ++k) s_part[(threadIdx.x >> 5) * 8 + k] = v[k];
-  }
-  __device__ __forceinline__ void load(const int* s_part, int warps) {
-    for (int w = 0; w < warps; ++w) {
-      rmax = max(rmax, s_part[w * 8]);
-      rmin = min(rmin, s_part[w * 8 + 1]);
-      emax = max(emax, s_part[w * 8 + 2]);
-      emin = min(emin, s_part[w * 8 + 3]);
-      mmax = max(mmax, s_part[w * 8 + 4]);
-    }
-  }
-  // density and energy positive and within kFixRange binades each, nothing huge or non-finite
-  __device__ __forceinline__ bool fits() const {
-    return rmin > 0 && emin > 0 && exp_of(rmax) - exp_of(rmin) <= kFixRange &&
-           exp_of(emax) - exp_of(emin) <= kFixRange &&
-           max(exp_of(rmax), max(exp_of(emax), exp_of(mmax))) <= kFixMaxExp;
-  }
-};
-
 // Whether most of a cell's energy is kinetic (p' = E - |m|^2 / (2 rho) below 2^-9 E) or its values lie
 // beyond 2^+-60: p' then amplifies the rounding of a state by E / p', the strengths of a fast, even
-// stream are that rounding, and the tile keeps to FP64.  From the high words of rho, m, E; in
-// FP32, whose few units in 2^-20 do not matter to the rule.
+// stream are that rounding, and the stencils that hold the cell keep to FP64.  From the high words of
+// rho, m, E; in FP32, whose few units in 2^-20 do not matter to the rule, the two momenta alike.
 __device__ __forceinline__ bool fix_fast(int rho, int mx, int my, int e) {
   auto f = [](int hi) {  // |x| truncated to 20 bits (0 below 2^-63)
     const int b = (hi & 0x7fffffff) - (896 << 20);
@@ -379,7 +282,7 @@ __device__ __forceinline__ bool fix_fast(int rho, int mx, int my, int e) {
   };
   const float r = f(rho), u = f(mx), v = f(my), en = f(e);
   return !(r > 0.0f && en > 0.0f && fmaxf(fmaxf(r, en), fmaxf(u, v)) < 1e18f) ||
-         u * u + v * v > 2.0f * (1.0f - 1.0f / 512.0f) * r * en;
+         __fadd_rn(__fmul_rn(u, u), __fmul_rn(v, v)) > 2.0f * (1.0f - 1.0f / 512.0f) * r * en;
 }
 
 // One tile: faces a0 .. a0+TN-1 along the sweep on lines b0 .. b0+tt-1, 1 <= tt <= TT
@@ -387,18 +290,14 @@ __device__ __forceinline__ bool fix_fast(int rho, int mx, int my, int e) {
 // laid out for TT lines whatever tt is.
 //
 // 2D flows with a front in both directions (some x-face and some y-face strength beyond smooth_limit,
-// below which every branch is linear) take both reconstructions in fixed point on the integer units
-// (ase_df_fixed.cuh) in the tiles whose density and energy span few binades (TileSpan::fits,
-// fix_fast),
-// wherever the branch is the linear one of order R; the FP64 pipe is left to the Gauss points.
-// The other branches run in FP64 in second passes over queues of such cells and faces.  Normal
-// values are then kept in shared memory as limbs at the tile's exponents.  An order-9 face then
-// takes 287 FP64 instructions instead of 586 (pipe 72 % busy, the rest waits on the 16 resident
-// warps); 187 since the products of the Gauss points left the pipe as well (ase_df_imul.cuh).  Measured
-// before that, FP64 -> fixed point: Configuration 3 512^2 order 5, one step, 1350 -> 1013 us;
-// the 1600 x 800 order-9 jet residual 3700 -> 2653 us; 64 mixed problems 14.5 -> 11.1 ms.  Exponents
-// per line with aligned sums measured 1046 / 2708 us / 13.0 ms: the alignment costs instructions,
-// and lines crossing a strong front made their tiles slower than plain FP64.
+// below which every branch is linear) take the linear branch of order R of both reconstructions in
+// fixed point on the integer units (ase_df_fixed.cuh), stencil by stencil where its values span few
+// binades and no cell of it is fast (fix_fast); the FP64 pipe is left to the Gauss points.  What a
+// face gets depends on its own stencils alone, not on the tile.  The other branches run in FP64
+// in second passes over queues of such cells and faces.
+// FP64 -> fixed point: Configuration 3 512^2 order 5, one step, 1267 -> 1032 us; the 1600 x 800 order-9 jet
+// residual 3580 -> 2403 us; 64 mixed problems 13.1 -> 10.3 ms.  One exponent per tile measured 950 us, 2410 us and 10.6
+// ms: it converts a value once, but cuts off the digits of values far below the tile's largest.
 // Flows without a front in both directions stay in FP64 to the bit: their strengths are differences of two
 // reconstructions that agree to rounding (1e-12 made of 1e-16 parts on a fine smooth grid), so
 // any other rounding of a state, however exact, shows in the fifth digit of the strengths; with a
@@ -443,12 +342,8 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   int* s_queue = reinterpret_cast<int*>(smem + TL::queue_offset);
   unsigned int* s_qn = reinterpret_cast<unsigned int*>(s_queue + TL::QCAP);
   if (tid < 2) s_qn[tid] = 0u;
-  // fixed point: a flag for a value that does not fit, and the warps' spans
-  int* s_any = reinterpret_cast<int*>(smem + TL::span_offset);
-  int* s_part = s_any + 2;
-  if (DIM == 2 && tid == 0) *s_any = 0;
-  Limbs* iQP = reinterpret_cast<Limbs*>(sQP);
-  Limbs* iQM = reinterpret_cast<Limbs*>(sQM);
+  // fixed point: the fast cells of the staged lines (bit aa of word bb), then of each line's 2K+1 lines
+  unsigned int* s_fast = reinterpret_cast<unsigned int*>(smem + TL::fast_offset);
   const bool front = DIM == 2 && args.front != nullptr && args.front[0] != 0u && args.front[1] != 0u;
   const unsigned long long limit = smooth_limit(g.thres);
   // ---- staging: consecutive threads take consecutive addresses along the direction in which the
@@ -459,7 +354,6 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   // a tile whose halo lies inside the grid needs none of the boundary's index maps
   const bool inside = DIM == 2 && a0 - 1 - K >= 0 && a0 + TN - 1 + K < n && b0 - KT >= 0 && b0 + tt + KT <= mlin;
   // cell averages: cells a0-1-K .. a0+TN-1+K, lines b0-KT .. b0+tt+KT-1
-  TileSpan span;
   // (16-line tiles: one component of a cell per thread, which loads one value instead of four in turn)
   const int staged = nb * NA;
   for (int k = tid; k < (TL::split ? C * staged : staged); k += NT) {
@@ -474,40 +368,18 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       const double* src = args.W + (size_t)b * stb + (size_t)a * sta;
 #pragma unroll kLU
       for (int c = c0; c < cn; ++c) {
-        const double v = __ldg(src + (size_t)c * g.nx * g.ny);
-        dst[c * NB * NA] = v;
-        if (DIM == 2) span.add(c, C - 1, v);
+        dst[c * NB * NA] = __ldg(src + (size_t)c * g.nx * g.ny);
       }
     } else {
       const int i = (DIR == 0) ? a : b, j = (DIR == 0) ? b : a;
 #pragma unroll 1
       for (int c = c0; c < cn; ++c) {
-        const double v = fetch_w(g, args.W, c, i, j, ts);
-        dst[c * NB * NA] = v;
-        if (DIM == 2) span.add(c, C - 1, v);
+        dst[c * NB * NA] = fetch_w(g, args.W, c, i, j, ts);
       }
     }
   }
-  bool fast = false;  // a staged cell that asks for FP64 (fix_fast)
-  if (front) {
-    if constexpr (DIM == 2 && TT == 32) {
-      // a tile of 32 lines takes the exponents of the 64-line tile it is half of, so that the tile
-      // shape does not change the results: the other half's lines are looked at, not staged
-      const int bx = (b0 & 32) ? b0 - 32 - KT : b0 + 32 + KT;
-      for (int idx = tid; idx < 32 * NA; idx += NT) {
-        const int a = a0 - 1 - K + ((DIR == 0) ? idx % NA : idx / 32), b = bx + ((DIR == 0) ? idx / NA : idx % 32);
-        int hi[C];
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-          const double v = (DIR == 0) ? fetch_w(g, args.W, c, a, b, ts) : fetch_w(g, args.W, c, b, a, ts);
-          span.add(c, C - 1, v);
-          hi[c] = (int)(dbits(v) >> 32);
-        }
-        fast |= fix_fast(hi[0], hi[1], hi[2], hi[3]);
-      }
-    }
-    span.store(s_part);
-  }
+  if (front)
+    for (int bb = tid; bb < nb; bb += NT) s_fast[bb] = 0u;
   bool rough = false;  // a strength beyond the limit below which every branch is linear of order R
   // normal face strengths: faces a0-K .. a0+TN-1+K of every staged line
   for (int idx = tid; idx < nb * NSN; idx += NT) {
@@ -545,65 +417,32 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   // Interior cells serve a face on each side and are evaluated at both xi = 0 and xi = -1; the
   // two end cells serve one tile face each (qa = 0: its xi = 0 value, the left state of face
   // a0; qa = NQ-1: its xi = -1 value).
-  bool fixed = false;
-  int ex[3];  // exponents of density, momentum, energy
-  if (front) {
-    span.load(s_part, NT / 32);
-    if constexpr (DIM == 2) {
+  bool fast = false;  // whether a staged cell is fast
+  if constexpr (DIM == 2) {
+    if (front) {
       const int* hi = reinterpret_cast<const int*>(sW) + 1;
       for (int idx = tid; idx < nb * NA; idx += NT)
-        fast |= fix_fast(hi[2 * idx], hi[2 * (NB * NA + idx)], hi[2 * (2 * NB * NA + idx)], hi[2 * (3 * NB * NA + idx)]);
-    }
-    fixed = !__syncthreads_or(fast) && span.fits();
-    ex[0] = fix_exponent(exp_of(span.rmax));
-    ex[1] = fix_exponent(exp_of(span.mmax));
-    ex[2] = fix_exponent(exp_of(span.emax));
-  }
-  auto comp_exp = [&](int c) { return c == 0 ? ex[0] : c == C - 1 ? ex[2] : ex[1]; };
-  if (fixed) {
-    for (int it = tid; it < C * nb; it += NT) {
-      int c, bb;
-      dnb.split(it, c, bb);
-      const int row = c * NB + bb;
-      fix_line<R, NA, NQ>(sW + row * NA, comp_exp(c), iQP + row * NQ, iQM + row * NQ);
-    }
-    if (rough)
-      for (int it = tid; it < NQ * nb; it += NT)
-        defer_item(select_branch<R>(sSn + (it / NQ) * NSN + it % NQ, g.thres).m != R, it, s_queue, &s_qn[0]);
-    __syncthreads();
-    // cells of another branch, in FP64, then converted
-    const int nq = (int)s_qn[0];
-    if (nq > 0) {
-      const int cs = nq * C <= NT ? C : 1;  // threads per cell (as below)
-      for (int k = tid; k < nq * cs; k += NT) {
-        const int it = s_queue[k / cs];
-        const int bb = it / NQ, qa = it % NQ;
-        const Branch br = select_branch<R>(sSn + bb * NSN + qa, g.thres);
-#pragma unroll 1
-        for (int c = k % cs; c < C; c += cs) {
-          const int row = c * NB + bb, e = comp_exp(c);
-          double out[2];
-          recon_eval<R, 2>(sW + row * NA + qa + K, 1, br, T, 0, out);
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            if (exp_of((int)(dbits(out[q]) >> 32) & 0x7fffffff) > e + 1) *s_any = 1;  // e.g. non-finite
-            else (q == 0 ? iQP : iQM)[row * NQ + qa] = fix_split(fix_join(fix_from_double(out[q], e)));
-          }
+        if (fix_fast(hi[2 * idx], hi[2 * (NB * NA + idx)], hi[2 * (2 * NB * NA + idx)], hi[2 * (3 * NB * NA + idx)])) {
+          atomicOr(&s_fast[idx / NA], 1u << idx % NA);
+          fast = true;
         }
-      }
-      __syncthreads();
-      if (*s_any) {  // the whole tile in FP64
-        fixed = false;
-        __syncthreads();
-        if (tid == 0) s_qn[0] = 0u;
-        __syncthreads();
-      }
+      fast = __syncthreads_or(fast);
+      if (fast)  // read after phase 1
+        for (int tb = tid; tb < tt; tb += NT) {
+          unsigned int m = 0u;
+          for (int l = 0; l <= 2 * K; ++l) m |= s_fast[tb + l];
+          s_fast[NB + tb] = m;
+        }
     }
   }
-  if (!fixed) {
-    // FP64: the end cells come last in the work list and evaluate one point; fallback cells are
-    // deferred (defer_item) and done in a second pass.  A 16-line tile without a branch choice
-    // gives each component of a cell a thread.
+  // fixed point for a stencil that starts at staged cell qa of line (of lines) k, of branch m
+  auto fixed = [&](int m, int k, int qa) {
+    return front && m == R && !(fast && (s_fast[k] >> qa & ((1u << (2 * K + 1)) - 1u)) != 0u);
+  };
+  {
+    // The end cells come last in the work list and evaluate one point; fallback cells (in a flow with a
+    // front: those of any branch but the order-R linear one) are deferred (defer_item) and done in a
+    // second pass.  A 16-line tile without a branch choice gives each component of a cell a thread.
     const bool comps = TL::split && !rough;
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
@@ -622,13 +461,15 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
           qa = pt * (NQ - 1);
         }
         const Branch br = branch(sSn + bb * NSN + qa);
-        if (R >= 5 && rough && pass == 0 && defer_item(br.m == 0, it, s_queue, &s_qn[0])) continue;
+        if ((R >= 5 || front) && rough && pass == 0 &&
+            defer_item(front ? br.m != R : br.m == 0, it, s_queue, &s_qn[0])) continue;
+        const bool fix = fixed(br.m, bb, qa);
         if (pt < 0) {
 #pragma unroll kCU
           for (int c = c0; c < cn; ++c) {
             const double* v = sW + (c * NB + bb) * NA + qa + K;  // W_0 of this cell
             double out[2];
-            recon_eval<R, 2>(v, 1, br, T, 0, out);
+            if (DIM == 1 || !(fix && fix_normal<R, 2>(v, 1, out))) recon_eval<R, 2>(v, 1, br, T, 0, out);
             sQP[(c * NB + bb) * NQ + qa] = out[0];
             sQM[(c * NB + bb) * NQ + qa] = out[1];
           }
@@ -638,13 +479,13 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
           for (int c = c0; c < cn; ++c) {
             const double* v = sW + (c * NB + bb) * NA + qa + K;
             double out[1];
-            recon_eval<R, 1>(v, 1, br, T, pt, out);
+            if (DIM == 1 || !(fix && fix_normal<R, 1>(v, pt ? -1 : 1, out))) recon_eval<R, 1>(v, 1, br, T, pt, out);
             dst[(c * NB + bb) * NQ + qa] = out[0];
           }
         }
       }
       __syncthreads();  // pass 0: the queue is complete; last pass: phase 1 is done
-      if (R < 5 || s_qn[0] == 0u || pass == 1) break;
+      if (s_qn[0] == 0u || pass == 1) break;
       const int nq = (int)s_qn[0];
       if (nq * C > NT) continue;
       // a short queue: one component of a cell per thread.  The fallback of one component is some
@@ -671,26 +512,15 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
     }
   }
 
-  // Gauss-point values of component cs / 2 of the state on side cs % 2 of a face, its branch bt;
-  // fixed point: in FP64 from the limbs where a side of the face has another branch (lin: none has)
-  auto tang_point = [&](int cs, int fa, int tb, const Branch& bt, bool lin, double* out) {
-    const int c = cs >> 1, side = cs & 1;
-    const int at = (c * NB + tb) * NQ + fa + side;  // line -K of the stencil
-    if (!fixed) {
-      tang_eval<R, G>((side == 0 ? sQP : sQM) + at + K * NQ, NQ, bt, T, out);
-    } else if (lin) {
-      fix_gauss<R, G, NQ>((side == 0 ? iQP : iQM) + at + K * NQ, comp_exp(c), out);
-    } else {
-      double v[2 * K + 1];
-#pragma unroll
-      for (int t = 0; t <= 2 * K; ++t)
-        v[t] = fix_to_double(fix_join((side == 0 ? iQP : iQM)[at + t * NQ]), comp_exp(c));
-      tang_eval<R, G>(v + K, 1, bt, T, out);
-    }
+  // Gauss-point values of component cs / 2 of the state on side cs % 2 of a face, its branch bt
+  auto tang_point = [&](int cs, int fa, int tb, const Branch& bt, double* out) {
+    const int qa = fa + (cs & 1);
+    const double* v = ((cs & 1) == 0 ? sQP : sQM) + ((cs >> 1) * NB + tb + K) * NQ + qa;
+    if (DIM == 1 || !(fixed(bt.m, NB + tb, qa) && fix_gauss<R, G>(v, NQ, out))) tang_eval<R, G>(v, NQ, bt, T, out);
   };
   // ---- phase 2: faces ----
-  // 2D: faces with a fallback tangential reconstruction on either side (fixed point: with any but
-  // the order-R linear one) are deferred.
+  // 2D: faces with a fallback tangential reconstruction on either side (in a flow with a front: with any
+  // but the order-R linear one) are deferred.
   if constexpr (TL::split) {
     // Tiles of up to 16 lines, on grids that give an SM one or two of them: a face per thread would
     // leave half or more of the CTA idle while a quarter of the SM's FP64 unit works on chains of some
@@ -725,7 +555,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         if (rough) bt = sB[tb * NQ + fa + (cs & 1)];
         if (rough && pass == 0) {
           const int m2 = sB[tb * NQ + fa + 1 - (cs & 1)].m;  // the other side's
-          const bool later = fixed ? bt.m != R || m2 != R : R >= 5 && (bt.m == 0 || m2 == 0);
+          const bool later = front ? bt.m != R || m2 != R : R >= 5 && (bt.m == 0 || m2 == 0);
           if (defer_item(later && cs == 0, it, s_queue, &s_qn[1]) || later) continue;
         }
         if (counting && cs < 2) {
@@ -733,7 +563,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
           atomicAdd(&hist_s[branch_slot(bt.m)], 1u);
         }
         double out[G];
-        tang_point(cs, fa, tb, bt, pass == 0, out);
+        tang_point(cs, fa, tb, bt, out);
 #pragma unroll
         for (int q = 0; q < G; ++q) sP[(((cs & 1) * G + q) * C + (cs >> 1)) * NF + it] = out[q];
       }
@@ -807,7 +637,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         bt[0] = branch(sSt + fa * NST + tb);  // the columns of the two states
         bt[1] = branch(sSt + (fa + 1) * NST + tb);
         if (rough && pass == 0) {
-          const bool defer = fixed ? bt[0].m != R || bt[1].m != R : R >= 5 && (bt[0].m == 0 || bt[1].m == 0);
+          const bool defer = front ? bt[0].m != R || bt[1].m != R : R >= 5 && (bt[0].m == 0 || bt[1].m == 0);
           if (defer_item(defer, it, s_queue, &s_qn[1])) continue;
         }
       }
@@ -825,7 +655,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
 #pragma unroll 1
         for (int cs = 0; cs < 2 * C; ++cs) {
           double out[G];
-          tang_point(cs, fa, tb, (cs & 1) == 0 ? bt[0] : bt[1], pass == 0, out);
+          tang_point(cs, fa, tb, (cs & 1) == 0 ? bt[0] : bt[1], out);
 #pragma unroll
           for (int q = 0; q < G; ++q) st[cs & 1][q][cs >> 1] = out[q];
         }
