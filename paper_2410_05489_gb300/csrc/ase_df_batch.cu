@@ -36,6 +36,7 @@ namespace {
 struct BatchProblem {
   GridInfo g;
   int ndim, variant;        // variant = (ndim - 1) * 4 + (order - 3) / 2
+  int front;                // looks_for_front: the rule of the problem alone, and so its bits
   long long w_off, sx_off, sy_off, fx_off, fy_off, cell_off;
   double inv_dx, inv_dy, cfl, t_end, inflow_speed;
 };
@@ -129,8 +130,8 @@ batch_sweep_kernel(const BatchProblem* __restrict__ probs, const int4* __restric
     a.F = (DIR == 0) ? P.Fx + pb.fx_off : P.Fy + pb.fy_off;
     a.s_out = (DIR == 0) ? sp.sxout : sp.syout;
     a.st = states + w.x;
-    if (stage > 0) a.front = a.st->front[stage - 1];  // read for 2D problems only
-    if (stage == 1 || stage == 2) a.front_out = &a.st->front[stage][DIR];
+    if (pb.front && stage > 0) a.front = a.st->front[stage - 1];
+    if (pb.front && (stage == 1 || stage == 2)) a.front_out = &a.st->front[stage][DIR];
     if (DIR == 0 && w.y == 0 && w.z == 0 && threadIdx.x <= kRepairPasses) {
       a.st->cnt[threadIdx.x] = 0u;  // repair counters of this problem's stage
       a.st->rbad[threadIdx.x] = 0u;
@@ -205,7 +206,7 @@ __device__ __forceinline__ RepairArgs repair_args(const BatchPtrs& P, const Batc
   r.dt_fixed = 0.0;
   r.stage = stage;
   r.pass = pass;
-  if (stage < 3) r.front_out = st->front[stage];
+  if (pb.front && stage < 3) r.front_out = st->front[stage];
   return r;
 }
 
@@ -243,6 +244,7 @@ __global__ void __launch_bounds__(256) batch_max_speed_kernel(const BatchProblem
       continue;
     }
     max_speed_range<2>(pb.g, a, first, (size_t)ch.z, blockDim.x);
+    if (!pb.front) continue;
     // the same share of the strengths, the last chunk also the ny (nx) entries past the cell count
     const size_t ncell = (size_t)pb.g.nx * pb.g.ny;
     const bool tail = (size_t)ch.z == ncell;
@@ -387,6 +389,7 @@ static void fill_grid(const ase_df_params& p, BatchProblem& d) {
   g.gg1 = p.gamma * (p.gamma - 1.0);
   g.thres = p.sigma_thres;
   d.ndim = p.ndim;
+  d.front = looks_for_front(p.ndim, g, p.order);
   d.variant = (p.ndim - 1) * 4 + (p.order - 3) / 2;
   d.cfl = p.cfl;
   d.t_end = p.t_end;

@@ -73,3 +73,31 @@ def test_uniform_gas_beside_a_front(A, order):  # noqa: F811
     far = np.ones((n, n), bool)
     far[120 - order:170 + order, 90 - order:160 + order] = False
     assert np.all(L.cpu().numpy()[:, far] == 0.0)
+
+@pytest.mark.parametrize("order", [3, 5, 7, 9])
+def test_tiles_and_launches_do_not_change_the_bits(A, order):  # noqa: F811
+    """Batched (8 x 64 and 8 x 32 tiles) and alone (the planned tiles): the same strengths and states."""
+    from paper_2410_05489_gb300 import batch
+
+    shapes = [(64, 64), (100, 90), (128, 128), (150, 141), (210, 200), (300, 270)]
+    probs = [P.riemann_2d(m, order, 3 * order + m, ny=k) for m, k in shapes]
+    out = []
+    for lines in (64, 32):
+        bt = batch.Batch([p for p, _ in probs], [w for _, w in probs])
+        try:
+            bt.set_tiles((lines,) * 4)
+            bt.run(2)
+            out.append([(bt.state(i), *bt.sigma(i)) for i in range(len(probs))])
+        finally:
+            bt.close()
+    for i, (pb, W) in enumerate(probs):
+        s = A.Solver(pb, W)
+        try:
+            s.step()
+            s.step()
+            alone = [t.cpu().numpy() for t in (s.W, s.sx, s.sy)]
+        finally:
+            s.close()
+        for a, b, c in zip(out[0][i], out[1][i], alone):
+            assert np.array_equal(a, b)
+            assert np.array_equal(a, c), (shapes[i], np.abs(a - c).max())
