@@ -222,10 +222,12 @@ cudaError_t launch_sweep_r9(int dim, int dir, const GridInfo& g, const SweepArgs
 cudaError_t launch_combine(int dim, const GridInfo& g, const CombineArgs& a, cudaStream_t s);
 cudaError_t launch_max_speed(int dim, const GridInfo& g, const SpeedArgs& a, cudaStream_t s);
 // Single 2D problems below this many cells keep to FP64: a step is bound by its chain of launches
-// there, and looking for a front costs what the fixed-point sweep gains.
-constexpr long long kFrontCells = 128 * 128, kFrontCells3 = 200 * 200;
+// there, and looking for a front costs what the fixed-point sweep gains.  Order 3 keeps to FP64
+// at every size: its stencils of three cells gain 8 % of a 1024^2 Riemann residual (513 -> 472 us), and
+// the code alone costs the smooth one 6 % (501 -> 530 us) and 48^2 - 128^2 runs as much.
+constexpr long long kFrontCells = 128 * 128;
 inline bool looks_for_front(int dim, const GridInfo& g, int order) {
-  return dim == 2 && (long long)g.nx * g.ny >= (order == 3 ? kFrontCells3 : kFrontCells);
+  return dim == 2 && order >= 5 && (long long)g.nx * g.ny >= kFrontCells;
 }
 // front[0] of the status word from the strengths a 2D stage consumes.
 cudaError_t launch_strength(const GridInfo& g, const double* sx, const double* sy, DevState* st, cudaStream_t s);

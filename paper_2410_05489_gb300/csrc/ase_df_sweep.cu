@@ -11,7 +11,7 @@
 //            (r-1)/2 Gauss points (Sec. 2.1, Remark 2 of Sec. 3.1), the local
 //            Lax-Friedrichs flux and the discontinuity strength per Gauss point
 //            (Sec. 2.3, Sec. 3.1), the Gauss-weighted face flux and the face sigma.
-// In flows with a front the linear reconstructions of both phases run in fixed point on the
+// In flows with a front the linear reconstructions (from order 5) of both phases run in fixed point on the
 // integer units (ase_df_fixed.cuh, sweep_tile).
 // The face fluxes go to global memory; the flux difference and the RK combination are
 // done by the combine kernel.
@@ -89,8 +89,13 @@ cudaError_t launch(const GridInfo& g, const SweepArgs& a, const Tables& t, cudaS
         p = p8;
         tiles = tiles8;
       }
-      // tiles of at most 16 lines: several threads a face (sweep_tile)
-      if ((m + p.nb_lo - 1) / p.nb_lo <= 16) return launch_grid<R, DIM, DIR, 16, true>(g, a, t, s, dim3((unsigned)tiles), p);
+      // tiles of at most 16 lines: several threads a face (sweep_tile).  Not at order 3 where tiles of more than
+      // 8 lines of both sweeps fit in one wave: its short stencils leave little to split, and two barriers are
+      // dearer (4 steps of Riemann data: 96^2 291 -> 278 us, 112^2 324 -> 307, 128^2 327 -> 313; at 8 lines, 64^2, or in
+      // two waves, 160^2, the split tile is the faster: 245 against 277, 370 against 421).
+      const int lines = (m + p.nb_lo - 1) / p.nb_lo;
+      if (lines <= 16 && !(R == 3 && lines > 8 && 2 * tiles <= slots))
+        return launch_grid<R, DIM, DIR, 16, true>(g, a, t, s, dim3((unsigned)tiles), p);
       return launch_grid<R, DIM, DIR, TT, true>(g, a, t, s, dim3((unsigned)tiles), p);
     }
     if (cols > 0x7fffffffLL || q > 65535) return cudaErrorInvalidConfiguration;

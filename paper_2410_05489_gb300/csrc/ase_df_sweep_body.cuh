@@ -289,7 +289,7 @@ __device__ __forceinline__ bool fix_fast(int rho, int mx, int my, int e) {
 // (threadIdx.x is the worker index); smem holds Tile<R, DIM, TT>::sweep_doubles doubles,
 // laid out for TT lines whatever tt is.
 //
-// 2D flows with a front in both directions (some x-face and some y-face strength beyond smooth_limit,
+// 2D flows of order 5 and more with a front in both directions (some x-face and some y-face strength beyond smooth_limit,
 // below which every branch is linear) take the linear branch of order R of both reconstructions in
 // fixed point on the integer units (ase_df_fixed.cuh), stencil by stencil where its values span few
 // binades and no cell of it is fast (fix_fast); the FP64 pipe is left to the Gauss points.  What a
@@ -315,7 +315,10 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   // the branches of all components and two forms of four points made 760 KB of code, far beyond
   // the instruction cache (245 KB rolled; 64^2 order-7 run of 4 steps 435 -> 404 us).  1D unrolls its
   // components: there the chain of one cell bounds the tile.
-  constexpr int kCU = (DIM == 1) ? C : 1, kLU = TL::split ? 1 : C;
+  // So do 64-line tiles of order 3, whose branches are short: 4 steps at 230^2 582 -> 549 us, 256^2 650 -> 632;
+  // a 1024^2 residual 497 -> 501.
+  constexpr bool kFix = DIM == 2 && R >= 5;  // fixed point (ase_df_fixed.cuh)
+  constexpr int kCU = (DIM == 1 || (R == 3 && !TL::split)) ? C : 1, kLU = TL::split ? 1 : C;
   // Products of the Gauss points on the integer units (ase_df_imul.cuh), where the tile has the
   // warps to fill the FP64 pipe: the 1024^2 order-9 step 7393 -> 6466 us, the 65537-cell order-9
   // residual 41.1 -> 39.0 us.  The 32-thread tiles and those of up to 8 lines (two CTAs of a few warps'
@@ -344,7 +347,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   if (tid < 2) s_qn[tid] = 0u;
   // fixed point: the fast cells of the staged lines (bit aa of word bb), then of each line's 2K+1 lines
   unsigned int* s_fast = reinterpret_cast<unsigned int*>(smem + TL::fast_offset);
-  const bool front = DIM == 2 && args.front != nullptr && args.front[0] != 0u && args.front[1] != 0u;
+  const bool front = kFix && args.front != nullptr && args.front[0] != 0u && args.front[1] != 0u;
   const unsigned long long limit = smooth_limit(g.thres);
   // ---- staging: consecutive threads take consecutive addresses along the direction in which the
   // arrays are contiguous (the sweep for x-faces, the lines for y-faces) ----
@@ -418,7 +421,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   // two end cells serve one tile face each (qa = 0: its xi = 0 value, the left state of face
   // a0; qa = NQ-1: its xi = -1 value).
   bool fast = false;  // whether a staged cell is fast
-  if constexpr (DIM == 2) {
+  if constexpr (kFix) {
     if (front) {
       const int* hi = reinterpret_cast<const int*>(sW) + 1;
       for (int idx = tid; idx < nb * NA; idx += NT)
@@ -461,15 +464,15 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
           qa = pt * (NQ - 1);
         }
         const Branch br = branch(sSn + bb * NSN + qa);
-        if ((R >= 5 || front) && rough && pass == 0 &&
-            defer_item(front ? br.m != R : br.m == 0, it, s_queue, &s_qn[0])) continue;
+        if (R >= 5 && rough && pass == 0 && defer_item(front ? br.m != R : br.m == 0, it, s_queue, &s_qn[0]))
+          continue;
         const bool fix = fixed(br.m, bb, qa);
         if (pt < 0) {
 #pragma unroll kCU
           for (int c = c0; c < cn; ++c) {
             const double* v = sW + (c * NB + bb) * NA + qa + K;  // W_0 of this cell
             double out[2];
-            if (DIM == 1 || !(fix && fix_normal<R, 2>(v, 1, out))) recon_eval<R, 2>(v, 1, br, T, 0, out);
+            if (!kFix || !(fix && fix_normal<R, 2>(v, 1, out))) recon_eval<R, 2>(v, 1, br, T, 0, out);
             sQP[(c * NB + bb) * NQ + qa] = out[0];
             sQM[(c * NB + bb) * NQ + qa] = out[1];
           }
@@ -479,7 +482,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
           for (int c = c0; c < cn; ++c) {
             const double* v = sW + (c * NB + bb) * NA + qa + K;
             double out[1];
-            if (DIM == 1 || !(fix && fix_normal<R, 1>(v, pt ? -1 : 1, out))) recon_eval<R, 1>(v, 1, br, T, pt, out);
+            if (!kFix || !(fix && fix_normal<R, 1>(v, pt ? -1 : 1, out))) recon_eval<R, 1>(v, 1, br, T, pt, out);
             dst[(c * NB + bb) * NQ + qa] = out[0];
           }
         }
@@ -516,7 +519,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   auto tang_point = [&](int cs, int fa, int tb, const Branch& bt, double* out) {
     const int qa = fa + (cs & 1);
     const double* v = ((cs & 1) == 0 ? sQP : sQM) + ((cs >> 1) * NB + tb + K) * NQ + qa;
-    if (DIM == 1 || !(fixed(bt.m, NB + tb, qa) && fix_gauss<R, G>(v, NQ, out))) tang_eval<R, G>(v, NQ, bt, T, out);
+    if (!kFix || !(fixed(bt.m, NB + tb, qa) && fix_gauss<R, G>(v, NQ, out))) tang_eval<R, G>(v, NQ, bt, T, out);
   };
   // ---- phase 2: faces ----
   // 2D: faces with a fallback tangential reconstruction on either side (in a flow with a front: with any
@@ -555,7 +558,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         if (rough) bt = sB[tb * NQ + fa + (cs & 1)];
         if (rough && pass == 0) {
           const int m2 = sB[tb * NQ + fa + 1 - (cs & 1)].m;  // the other side's
-          const bool later = front ? bt.m != R || m2 != R : R >= 5 && (bt.m == 0 || m2 == 0);
+          const bool later = R >= 5 && (front ? bt.m != R || m2 != R : bt.m == 0 || m2 == 0);
           if (defer_item(later && cs == 0, it, s_queue, &s_qn[1]) || later) continue;
         }
         if (counting && cs < 2) {
@@ -616,7 +619,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         else args.F[((size_t)c * (g.ny + 1) + f) * g.nx + b] = sum;
       } else {
         const double sface = (G == 1) ? sum : sum * (1.0 / G);
-        if (args.front_out != nullptr && is_front(sface, limit)) *args.front_out = 1u;
+        if (kFix && args.front_out != nullptr && is_front(sface, limit)) *args.front_out = 1u;
         args.s_out[(DIR == 0) ? (size_t)b * (g.nx + 1) + f : (size_t)f * g.nx + b] = sface;
       }
     }
@@ -637,8 +640,8 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         bt[0] = branch(sSt + fa * NST + tb);  // the columns of the two states
         bt[1] = branch(sSt + (fa + 1) * NST + tb);
         if (rough && pass == 0) {
-          const bool defer = front ? bt[0].m != R || bt[1].m != R : R >= 5 && (bt[0].m == 0 || bt[1].m == 0);
-          if (defer_item(defer, it, s_queue, &s_qn[1])) continue;
+          const bool defer = front ? bt[0].m != R || bt[1].m != R : bt[0].m == 0 || bt[1].m == 0;
+          if (R >= 5 && defer_item(defer, it, s_queue, &s_qn[1])) continue;
         }
       }
       double st[2][G][C];
@@ -652,7 +655,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       }
       // left state: cell f-1 (plus face); right: cell f (minus face)
       if constexpr (DIM == 2) {
-#pragma unroll 1
+#pragma unroll (R == 3 ? 2 * C : 1)
         for (int cs = 0; cs < 2 * C; ++cs) {
           double out[G];
           tang_point(cs, fa, tb, (cs & 1) == 0 ? bt[0] : bt[1], out);
@@ -686,7 +689,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
         if (counting) atomicAdd(&hist_s[kBranchSlots - 1], nfb);
       }
       const double sface = (G == 1) ? ssum : ssum * (1.0 / G);
-      if (DIM == 2 && args.front_out != nullptr && is_front(sface, limit)) *args.front_out = 1u;
+      if (kFix && args.front_out != nullptr && is_front(sface, limit)) *args.front_out = 1u;
       if (DIR == 0) {
 #pragma unroll
         for (int c = 0; c < C; ++c) args.F[((size_t)c * g.ny + b) * (g.nx + 1) + f] = Fs[c];
