@@ -354,7 +354,7 @@ const char* ase_df_last_error(const ase_df_ctx* c) { return c ? c->err : g_init_
 static cudaError_t sweep(ase_df_ctx* c, int dir, const double* W, const double* sx, const double* sy,
                          double* F, double* s_out, cudaStream_t s, double tfrac, int stage, bool next) {
   SweepArgs a;
-  if (stage >= 0 && looks_for_front(c->dim, c->g, c->p.order)) {
+  if (stage >= 0 && looks_for_front(c->dim, c->g, c->p.order, stage == 0)) {
     a.front = c->st->front[stage > 0 ? stage - 1 : 0];
     if (next) a.front_out = &c->st->front[stage][dir];
   }
@@ -509,7 +509,8 @@ ase_df_status ase_df_residual(ase_df_ctx* c, const double* W, const double* sx_i
     return fail(c, ASE_DF_E_INVAL, "sigma_out must not alias sigma_in");
   cudaStream_t s = (cudaStream_t)stream;
   c->last_stream = s;
-  cudaError_t e = looks_for_front(c->dim, c->g, c->p.order) ? launch_strength(c->g, sx_in, sy_in, c->st, s) : cudaSuccess;
+  cudaError_t e = cudaSuccess;
+  if (looks_for_front(c->dim, c->g, c->p.order, true)) e = launch_strength(c->g, sx_in, sy_in, c->st, s);
   if (e == cudaSuccess) e = face_fluxes(c, W, sx_in, sy_in, sx_out, sy_out, s, 0, false);
   if (e != cudaSuccess) return cuda_fail(c, e, "residual sweep");
   e = combine(c, 0, W, W, L, 0.0, s, false);

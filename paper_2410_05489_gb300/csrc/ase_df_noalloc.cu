@@ -140,7 +140,7 @@ extern "C" ase_df_status ase_df_residual_noalloc(const ase_df_params* pin, const
 
   e = launch_state_kernel(st, 0, 0.0, s);  // clear the status word of the previous call
   if (e != cudaSuccess) return nfail(ASE_DF_E_CUDA, "status reset: %s", cudaGetErrorString(e));
-  const bool front = looks_for_front(p.ndim, g, p.order);
+  const bool front = looks_for_front(p.ndim, g, p.order, true);
   if (front && (e = launch_strength(g, sx_in, sy_in, st, s)) != cudaSuccess)
     return nfail(ASE_DF_E_CUDA, "strength reduction: %s", cudaGetErrorString(e));
   for (int dir = 0; dir < p.ndim; ++dir) {
