@@ -420,6 +420,7 @@ static cudaError_t combine(ase_df_ctx* c, int stage, const double* Wn, const dou
   a.Wn = Wn;
   a.Ws = Ws;
   a.out = out;
+  if (out == Wn) a.keep = c->W1;  // stage 3: W1 is no longer read
   a.st = c->st;
   a.inv_dx = c->inv_dx;
   a.inv_dy = c->inv_dy;
@@ -439,7 +440,7 @@ static cudaError_t combine(ase_df_ctx* c, int stage, const double* Wn, const dou
   r.mark = c->mark;
   r.Fx = c->Fx;
   r.Fy = c->Fy;
-  r.Wn = Wn;
+  r.Wn = a.keep != nullptr ? a.keep : Wn;
   r.Ws = Ws;
   r.out = out;
   r.sx_out = sxo;

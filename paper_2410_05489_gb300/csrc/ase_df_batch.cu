@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(256) batch_combine_kernel(const BatchProblem* 
     a.Wn = P.W + pb.w_off;
     a.Ws = sp.Ws;
     a.out = sp.out;
+    if (stage == 3) a.keep = P.W1 + pb.w_off;
     a.st = states + ch.x;
     a.inv_dx = pb.inv_dx;
     a.inv_dy = pb.inv_dy;
@@ -195,7 +196,7 @@ __device__ __forceinline__ RepairArgs repair_args(const BatchPtrs& P, const Batc
   r.mark = P.mark + pb.cell_off;
   r.Fx = P.Fx + pb.fx_off;
   r.Fy = P.Fy + pb.fy_off;
-  r.Wn = P.W + pb.w_off;
+  r.Wn = (stage == 3 ? P.W1 : P.W) + pb.w_off;  // stage 3's out is W: its combine keeps W^n in W1
   r.Ws = sp.Ws;
   r.out = sp.out;
   r.sx_out = sp.sxout;

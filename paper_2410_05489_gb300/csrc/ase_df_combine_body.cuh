@@ -94,7 +94,11 @@ __device__ __forceinline__ void combine_range(const GridInfo& g, const CombineAr
       if (a.stage == 0) q[c] = t;
       else if (a.stage == 1) q[c] = a.Ws[w] + t;
       else if (a.stage == 2) q[c] = fma(0.75, a.Wn[w], fma(0.25, a.Ws[w], t));
-      else q[c] = fma(1.0 / 3.0, a.Wn[w], fma(2.0 / 3.0, a.Ws[w], t));
+      else {
+        const double wn = a.Wn[w];
+        if (a.keep != nullptr) a.keep[w] = wn;
+        q[c] = fma(1.0 / 3.0, wn, fma(2.0 / 3.0, a.Ws[w], t));
+      }
       a.out[w] = q[c];
       if (!finite_bits(q[c])) bad = true;
     }

@@ -155,6 +155,7 @@ struct CombineArgs {
   const double* Wn;   // W^n
   const double* Ws;   // stage input W^(s)
   double* out;        // W^(s+1) (or L for stage 0)
+  double* keep = nullptr;  // stage 3, whose out overwrites Wn: takes a copy of Wn, for the repair
   DevState* st;
   double inv_dx, inv_dy;
   double dt_fixed;    // > 0: this dt; otherwise the CFL dt (stage 1 computes it)
