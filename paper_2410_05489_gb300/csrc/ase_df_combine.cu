@@ -94,7 +94,9 @@ __global__ void __launch_bounds__(256) repair_all_kernel(const GridInfo g, Repai
 
 // Combination and repair of one stage of a small 1D problem in one CTA, whose barrier takes the
 // place of the grid's.  Bound by latency: 200 cells take 4.3 us, 4.2 + 1.9 us and a launch gap as two
-// kernels.  Past 512 cells one SM's FP64 unit takes longer than the saved launch.
+// kernels.  Past some 400 cells one SM's FP64 unit takes longer than the saved launch: a step of a Sod tube
+// at order 5 in one launch and in two takes 41.3 and 45.3 us at 200 cells, 41.3 and 43.3 at 320, 45.4 and 46.6
+// at 400, 45.4 and 43.9 at 512.
 __global__ void __launch_bounds__(kSmallCells) combine_repair_kernel(const GridInfo g, const CombineArgs a,
                                                                      RepairArgs r) {
   const size_t first = threadIdx.x, stride = blockDim.x, ncell = (size_t)g.nx;

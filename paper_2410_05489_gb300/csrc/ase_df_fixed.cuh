@@ -1,10 +1,10 @@
 // Linear reconstructions in fixed point on the integer units.
 //
-// Why: this part issues FP64 at 1.6 lanes per cycle per SM (20 cycles a warp instruction,
-// whatever the operation) and 32 x 32 -> 64 bit multiply-adds at 54, beside each other.  The
+// Why: this part issues FP64 at 2 lanes per cycle per SM at most and 32 x 32 -> 64 bit
+// multiply-adds at 54, beside each other.  The
 // linear branches of Algorithm 1 are contractions of 3 to 9 cell averages with constant
-// weights, so they can leave the FP64 pipe to the Gauss-point flux: the 1024^2 order-9 sweep
-// spent 321 of its 586 FP64 instructions per face on them.
+// weights, so they can leave the FP64 pipe to the Gauss-point flux: of the 475 FP64 instructions
+// of an order-9 face in a smooth flow, whose products of the Gauss points run on the integer units, they are 321.
 //
 // The values of ONE stencil share one exponent e, that of the largest:
 //   |v| = M 2^(e - 1023 - 56), M < 2^57.

@@ -1,9 +1,8 @@
 // Products of doubles formed on the integer units, to the bit.
 //
-// Why: FP64 issues at 1.6 lanes per cycle per SM here, one instruction in 20 cycles of a warp
-// whatever it does.  A correctly rounded product takes four 32 x 32 -> 64 bit multiply-adds and
-// some 24 other integer instructions, about 0.4 cycles a lane beside an FP64 pipe that works on
-// (0.61 a lane).  So products that are no part of a fused multiply-add leave the FP64 pipe where
+// Why: FP64 issues at 2 lanes per cycle per SM at most here.  A correctly rounded product takes four
+// 32 x 32 -> 64 bit multiply-adds and some 24 other integer instructions, about 0.4 cycles a lane
+// beside an FP64 pipe that works on (0.5 to 0.6 a lane).  So products that are no part of a fused multiply-add leave the FP64 pipe where
 // it is the bound; where latency is (few warps on an SM), the FP64 instruction stays the shorter.
 #pragma once
 

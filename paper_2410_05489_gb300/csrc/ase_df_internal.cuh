@@ -239,7 +239,7 @@ cudaError_t launch_strength(const GridInfo& g, const double* sx, const double* s
 // when the stage update was physical everywhere; a grid barrier between passes).
 cudaError_t launch_repair_all(int dim, const GridInfo& g, const RepairArgs& a, cudaStream_t s);
 // Both of a 1D problem of at most kSmallCells cells in one launch of one CTA.
-constexpr int kSmallCells = 512;
+constexpr int kSmallCells = 416;
 cudaError_t launch_combine_repair(const GridInfo& g, const CombineArgs& a, const RepairArgs& r, cudaStream_t s);
 // A grid barrier that cannot complete (self-test of the bounded wait): raises
 // ASE_DF_FLAG_SYNC after about a second, then clears the barrier's arrival count.

@@ -289,12 +289,12 @@ __device__ __forceinline__ bool fix_fast(int rho, int mx, int my, int e) {
 // (threadIdx.x is the worker index); smem holds Tile<R, DIM, TT>::sweep_doubles doubles,
 // laid out for TT lines whatever tt is.
 //
-// 2D flows of order 5 and more with a front in both directions (some x-face and some y-face strength beyond smooth_limit,
-// below which every branch is linear) take the linear branch of order R of both reconstructions in
-// fixed point on the integer units (ase_df_fixed.cuh), stencil by stencil where its values span few
-// binades and no cell of it is fast (fix_fast); the FP64 pipe is left to the Gauss points.  What a
-// face gets depends on its own stencils alone, not on the tile.  The other branches run in FP64
-// in second passes over queues of such cells and faces.
+// 2D flows of order 5 and more with a front in both directions (some x-face and some y-face strength
+// beyond smooth_limit, below which every branch is linear) take the linear branch of order R of both
+// reconstructions in fixed point on the integer units (ase_df_fixed.cuh), stencil by stencil where its
+// values span few binades and no cell of it is fast (fix_fast); the FP64 pipe is left to the Gauss
+// points.  What a face gets depends on its own stencils alone, not on the tile.  The other branches
+// run in FP64 in second passes over queues of such cells and faces.
 // FP64 -> fixed point: Configuration 3 512^2 order 5, one step, 1267 -> 1032 us; the 1600 x 800 order-9 jet
 // residual 3580 -> 2403 us; 64 mixed problems 13.1 -> 10.3 ms.  One exponent per tile measured 950 us, 2410 us and 10.6
 // ms: it converts a value once, but cuts off the digits of values far below the tile's largest.
@@ -313,12 +313,13 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   constexpr int TI = (DIR == 0) ? 2 : 1;  // tangential momentum component
   // 2D loops over components and Gauss points stay rolled, their states in local memory: unrolled,
   // the branches of all components and two forms of four points made 760 KB of code, far beyond
-  // the instruction cache (245 KB rolled; 64^2 order-7 run of 4 steps 435 -> 404 us).  1D unrolls its
+  // the instruction cache (190 KB now; 64^2 order-7 run of 4 steps 435 -> 404 us).  1D unrolls its
   // components: there the chain of one cell bounds the tile.
   // So do 64-line tiles of order 3, whose branches are short: 4 steps at 230^2 582 -> 549 us, 256^2 650 -> 632;
   // a 1024^2 residual 497 -> 501.
   constexpr bool kFix = DIM == 2 && R >= 5;  // fixed point (ase_df_fixed.cuh)
-  constexpr int kCU = (DIM == 1 || (R == 3 && !TL::split)) ? C : 1, kLU = TL::split ? 1 : C;
+  constexpr bool kFlat = TL::split || NT == 32;
+  constexpr int kCU = (DIM == 1 || (R == 3 && !TL::split)) ? C : 1, kLU = kFlat ? 1 : C;
   // Products of the Gauss points on the integer units (ase_df_imul.cuh), where the tile has the
   // warps to fill the FP64 pipe: the 1024^2 order-9 step 7393 -> 6466 us, the 65537-cell order-9
   // residual 41.1 -> 39.0 us.  The 32-thread tiles and those of up to 8 lines (two CTAs of a few warps'
@@ -355,13 +356,14 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   const LineDiv dnb(nb);
   const int sta = (DIR == 0) ? 1 : g.nx, stb = (DIR == 0) ? g.nx : 1;
   // a tile whose halo lies inside the grid needs none of the boundary's index maps
-  const bool inside = DIM == 2 && a0 - 1 - K >= 0 && a0 + TN - 1 + K < n && b0 - KT >= 0 && b0 + tt + KT <= mlin;
+  const bool inside = a0 - 1 - K >= 0 && a0 + TN - 1 + K < n && (DIM == 1 || (b0 - KT >= 0 && b0 + tt + KT <= mlin));
   // cell averages: cells a0-1-K .. a0+TN-1+K, lines b0-KT .. b0+tt+KT-1
-  // (16-line tiles: one component of a cell per thread, which loads one value instead of four in turn)
+  // (16-line tiles and those of 32 threads: one component of a cell per thread, which loads one value instead
+  // of three or four in turn; a sweep of 2000 cells in 31-face tiles is 0.5 us shorter)
   const int staged = nb * NA;
-  for (int k = tid; k < (TL::split ? C * staged : staged); k += NT) {
-    const int c0 = TL::split ? (k >= staged) + (k >= 2 * staged) + (k >= 3 * staged) : 0;
-    const int cn = TL::split ? c0 + 1 : C, idx = k - c0 * staged;
+  for (int k = tid; k < (kFlat ? C * staged : staged); k += NT) {
+    const int c0 = kFlat ? (k >= staged) + (k >= 2 * staged) + (k >= 3 * staged) : 0;
+    const int cn = kFlat ? c0 + 1 : C, idx = k - c0 * staged;
     int bb, aa;
     if (DIR == 0) { aa = idx % NA; bb = idx / NA; }
     else dnb.split(idx, aa, bb);
@@ -375,7 +377,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       }
     } else {
       const int i = (DIR == 0) ? a : b, j = (DIR == 0) ? b : a;
-#pragma unroll 1
+#pragma unroll (DIM == 1 && !kFlat ? C : 1)
       for (int c = c0; c < cn; ++c) {
         dst[c * NB * NA] = fetch_w(g, args.W, c, i, j, ts);
       }
@@ -442,77 +444,79 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   auto fixed = [&](int m, int k, int qa) {
     return front && m == R && !(fast && (s_fast[k] >> qa & ((1u << (2 * K + 1)) - 1u)) != 0u);
   };
-  {
-    // The end cells come last in the work list and evaluate one point; fallback cells (in a flow with a
-    // front: those of any branch but the order-R linear one) are deferred (defer_item) and done in a
-    // second pass.  A 16-line tile without a branch choice gives each component of a cell a thread.
-    const bool comps = TL::split && !rough;
+  // The end cells come last in the work list and evaluate one point; fallback cells (in a flow with a
+  // front: those of any branch but the order-R linear one) are deferred (defer_item) and done in a
+  // second pass.  A 16-line tile without a branch choice gives each component of a cell a thread.
+  const bool comps = TL::split && !rough;
 #pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-      const int cells = NQ * nb;
-      const int count = (pass == 0) ? (comps ? C * cells : cells) : (int)s_qn[0];
-      for (int k = tid; k < count; k += NT) {
-        const int c0 = comps ? (k >= cells) + (k >= 2 * cells) + (k >= 3 * cells) : 0, cn = comps ? c0 + 1 : C;
-        const int it = (pass == 0) ? k - c0 * cells : s_queue[k];
-        int qa, bb, pt;  // pt -1: an interior cell, both points; 0 / 1: an end cell, one point
-        if (it < (NQ - 2) * nb) {
-          if (DIR == 0) { qa = 1 + it % (NQ - 2); bb = it / (NQ - 2); }
-          else { dnb.split(it, qa, bb); ++qa; }
-          pt = -1;
-        } else {
-          dnb.split(it - (NQ - 2) * nb, pt, bb);  // pt 0: cell qa = 0 at xi = 0; 1: qa = NQ-1 at xi = -1
-          qa = pt * (NQ - 1);
+  for (int pass = 0; pass < 2; ++pass) {
+    const int cells = NQ * nb;
+    const int count = (pass == 0) ? (comps ? C * cells : cells) : (int)s_qn[0];
+    for (int k = tid; k < count; k += NT) {
+      const int c0 = comps ? (k >= cells) + (k >= 2 * cells) + (k >= 3 * cells) : 0, cn = comps ? c0 + 1 : C;
+      const int it = (pass == 0) ? k - c0 * cells : s_queue[k];
+      int qa, bb, pt;  // pt -1: an interior cell, both points; 0 / 1: an end cell, one point
+      if (it < (NQ - 2) * nb) {
+        if (DIR == 0) { qa = 1 + it % (NQ - 2); bb = it / (NQ - 2); }
+        else { dnb.split(it, qa, bb); ++qa; }
+        pt = -1;
+      } else {
+        dnb.split(it - (NQ - 2) * nb, pt, bb);  // pt 0: cell qa = 0 at xi = 0; 1: qa = NQ-1 at xi = -1
+        qa = pt * (NQ - 1);
+        if (DIM == 1) pt = -1;  // both points: two of a warp's lanes would run a path of their own after the others'
+      }
+      const Branch br = branch(sSn + bb * NSN + qa);
+      if (R >= 5 && rough && pass == 0 && defer_item(front ? br.m != R : br.m == 0, it, s_queue, &s_qn[0]))
+        continue;
+      const bool fix = fixed(br.m, bb, qa);
+      if (pt < 0) {
+#pragma unroll kCU
+        for (int c = c0; c < cn; ++c) {
+          const double* v = sW + (c * NB + bb) * NA + qa + K;  // W_0 of this cell
+          double out[2];
+          if (!kFix || !(fix && fix_normal<R, 2>(v, 1, out))) recon_eval<R, 2>(v, 1, br, T, 0, out);
+          sQP[(c * NB + bb) * NQ + qa] = out[0];
+          sQM[(c * NB + bb) * NQ + qa] = out[1];
         }
-        const Branch br = branch(sSn + bb * NSN + qa);
-        if (R >= 5 && rough && pass == 0 && defer_item(front ? br.m != R : br.m == 0, it, s_queue, &s_qn[0]))
-          continue;
-        const bool fix = fixed(br.m, bb, qa);
-        if (pt < 0) {
+      } else {
+        double* dst = pt ? sQM : sQP;
 #pragma unroll kCU
-          for (int c = c0; c < cn; ++c) {
-            const double* v = sW + (c * NB + bb) * NA + qa + K;  // W_0 of this cell
-            double out[2];
-            if (!kFix || !(fix && fix_normal<R, 2>(v, 1, out))) recon_eval<R, 2>(v, 1, br, T, 0, out);
-            sQP[(c * NB + bb) * NQ + qa] = out[0];
-            sQM[(c * NB + bb) * NQ + qa] = out[1];
-          }
-        } else {
-          double* dst = pt ? sQM : sQP;
-#pragma unroll kCU
-          for (int c = c0; c < cn; ++c) {
-            const double* v = sW + (c * NB + bb) * NA + qa + K;
-            double out[1];
-            if (!kFix || !(fix && fix_normal<R, 1>(v, pt ? -1 : 1, out))) recon_eval<R, 1>(v, 1, br, T, pt, out);
-            dst[(c * NB + bb) * NQ + qa] = out[0];
-          }
+        for (int c = c0; c < cn; ++c) {
+          const double* v = sW + (c * NB + bb) * NA + qa + K;
+          double out[1];
+          if (!kFix || !(fix && fix_normal<R, 1>(v, pt ? -1 : 1, out))) recon_eval<R, 1>(v, 1, br, T, pt, out);
+          dst[(c * NB + bb) * NQ + qa] = out[0];
         }
       }
-      __syncthreads();  // pass 0: the queue is complete; last pass: phase 1 is done
-      if (s_qn[0] == 0u || pass == 1) break;
-      const int nq = (int)s_qn[0];
-      if (nq * C > NT) continue;
-      // a short queue: one component of a cell per thread.  The fallback of one component is some
-      // 200 dependent FP64 instructions, and the tile waits for its slowest thread (Sod tube of 200
-      // cells, first sweep 42.7 -> 19.6 us, later ones 11.7 -> 10.6); a long queue keeps one thread per cell, which chooses
-      // the branch (and divides for its DF factors) once.
-      for (int k = tid; k < nq * C; k += NT) {
-        const int it = s_queue[k / C], c = k % C;
-        int bb, qa;
-        if (it < (NQ - 2) * nb) {
-          if (DIR == 0) { qa = 1 + it % (NQ - 2); bb = it / (NQ - 2); }
-          else { dnb.split(it, qa, bb); ++qa; }
-        } else {
-          dnb.split(it - (NQ - 2) * nb, qa, bb);
-          qa *= NQ - 1;
-        }
-        double out[2];  // an end cell's value at its outer face is formed too and not read
-        recon_eval<R, 2>(sW + (c * NB + bb) * NA + qa + K, 1, select_branch<R>(sSn + bb * NSN + qa, g.thres), T, 0, out);
-        sQP[(c * NB + bb) * NQ + qa] = out[0];
-        sQM[(c * NB + bb) * NQ + qa] = out[1];
-      }
-      __syncthreads();
-      break;
     }
+    __syncthreads();  // pass 0: the queue is complete; last pass: phase 1 is done
+    if (s_qn[0] == 0u || pass == 1) break;
+    const int nq = (int)s_qn[0];
+    if (nq * C > NT) continue;
+    // a short queue: one component of a cell per thread.  The fallback of one component is some
+    // 200 dependent FP64 instructions, and the tile waits for its slowest thread (Sod tube of 200
+    // cells, first sweep 42.7 -> 19.6 us, later ones 11.7 -> 10.6); a long queue keeps one thread per cell, which chooses
+    // the branch (and divides for its DF factors) once.
+    for (int k = tid; k < nq * C; k += NT) {
+      const int it = s_queue[k / C], c = k % C;
+      int bb, qa;
+      if (it < (NQ - 2) * nb) {
+        if (DIR == 0) { qa = 1 + it % (NQ - 2); bb = it / (NQ - 2); }
+        else { dnb.split(it, qa, bb); ++qa; }
+      } else {
+        dnb.split(it - (NQ - 2) * nb, qa, bb);
+        qa *= NQ - 1;
+      }
+      double out[2];  // an end cell's value at its outer face is formed too and not read
+      const Branch br = select_branch<R>(sSn + bb * NSN + qa, g.thres);
+      const double* v = sW + (c * NB + bb) * NA + qa + K;
+      if (kFix) recon_eval<R, 2>(v, 1, br, T, 0, out);
+      else weno_eval<2>(v, 1, br, T, 0, out);  // 1D: nothing else is queued
+      sQP[(c * NB + bb) * NQ + qa] = out[0];
+      sQM[(c * NB + bb) * NQ + qa] = out[1];
+    }
+    __syncthreads();
+    break;
   }
 
   // Gauss-point values of component cs / 2 of the state on side cs % 2 of a face, its branch bt
