@@ -227,11 +227,11 @@ cudaError_t launch_max_speed(int dim, const GridInfo& g, const SpeedArgs& a, cud
 // at every size: its stencils of three cells gain 8 % of a 1024^2 Riemann residual (513 -> 472 us), and
 // the code alone costs the smooth one 6 % (501 -> 530 us) and 48^2 - 128^2 runs as much.
 // A step finds the front in its CFL kernel, or once for three stages; a residual needs a launch of its own,
-// 4 us, and looks from 256^2 cells (order 5, 128^2: smooth 35 against 38 us, Riemann data 133 both; 256^2: 84
-// against 88, 224 against 211).
-constexpr long long kFrontCells = 128 * 128, kFrontCellsResidual = 256 * 256;
+// 4 us, which order 5 pays back from 256^2 cells only (128^2: smooth 35 against 38 us, Riemann data 133 both;
+// 256^2: 84 against 88, 224 against 211; order 7, 160^2: 70 against 75, 202 against 169).
+constexpr long long kFrontCells = 128 * 128, kFrontCellsResidual5 = 256 * 256;
 inline bool looks_for_front(int dim, const GridInfo& g, int order, bool residual = false) {
-  return dim == 2 && order >= 5 && (long long)g.nx * g.ny >= (residual ? kFrontCellsResidual : kFrontCells);
+  return dim == 2 && order >= 5 && (long long)g.nx * g.ny >= (residual && order == 5 ? kFrontCellsResidual5 : kFrontCells);
 }
 // front[0] of the status word from the strengths a 2D stage consumes.
 cudaError_t launch_strength(const GridInfo& g, const double* sx, const double* sy, DevState* st, cudaStream_t s);
