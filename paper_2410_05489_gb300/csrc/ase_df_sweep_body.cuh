@@ -446,7 +446,8 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
   };
   // The end cells come last in the work list and evaluate one point; fallback cells (in a flow with a
   // front: those of any branch but the order-R linear one) are deferred (defer_item) and done in a
-  // second pass.  A 16-line tile without a branch choice gives each component of a cell a thread.
+  // second pass.  There, and in 1D, the end cells evaluate both points like the others, one of them not
+  // read: two lanes of a warp would run the same long chain once more after the others'.  A 16-line tile without a branch choice gives each component of a cell a thread.
   const bool comps = TL::split && !rough;
 #pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
@@ -463,7 +464,7 @@ __device__ __forceinline__ void sweep_tile(const GridInfo& g, const SweepArgs& a
       } else {
         dnb.split(it - (NQ - 2) * nb, pt, bb);  // pt 0: cell qa = 0 at xi = 0; 1: qa = NQ-1 at xi = -1
         qa = pt * (NQ - 1);
-        if (DIM == 1) pt = -1;  // both points: two of a warp's lanes would run a path of their own after the others'
+        if (DIM == 1 || pass == 1) pt = -1;  // both points (below)
       }
       const Branch br = branch(sSn + bb * NSN + qa);
       if (R >= 5 && rough && pass == 0 && defer_item(front ? br.m != R : br.m == 0, it, s_queue, &s_qn[0]))
