@@ -227,8 +227,8 @@ cudaError_t launch_max_speed(int dim, const GridInfo& g, const SpeedArgs& a, cud
 // at every size: its stencils of three cells gain 8 % of a 1024^2 Riemann residual (513 -> 472 us), and
 // the code alone costs the smooth one 6 % (501 -> 530 us) and 48^2 - 128^2 runs as much.
 // A step finds the front in its CFL kernel, or once for three stages; a residual needs a launch of its own,
-// 4 us, which order 5 pays back from 256^2 cells only (128^2: smooth 35 against 38 us, Riemann data 133 both;
-// 256^2: 84 against 88, 224 against 211; order 7, 160^2: 70 against 75, 202 against 169).
+// 4 us, which order 5 pays back from 256^2 cells only (128^2: smooth 34 against 38 us, Riemann data 111 both;
+// 256^2: 84 against 88, 214 against 195; order 7, 160^2: 71 against 75, 174 against 146).
 constexpr long long kFrontCells = 128 * 128, kFrontCellsResidual5 = 256 * 256;
 inline bool looks_for_front(int dim, const GridInfo& g, int order, bool residual = false) {
   return dim == 2 && order >= 5 && (long long)g.nx * g.ny >= (residual && order == 5 ? kFrontCellsResidual5 : kFrontCells);

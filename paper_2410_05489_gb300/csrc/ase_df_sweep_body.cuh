@@ -295,8 +295,8 @@ __device__ __forceinline__ bool fix_fast(int rho, int mx, int my, int e) {
 // values span few binades and no cell of it is fast (fix_fast); the FP64 pipe is left to the Gauss
 // points.  What a face gets depends on its own stencils alone, not on the tile.  The other branches
 // run in FP64 in second passes over queues of such cells and faces.
-// FP64 -> fixed point: Configuration 3 512^2 order 5, one step, 1267 -> 1032 us; the 1600 x 800 order-9 jet
-// residual 3580 -> 2403 us; 64 mixed problems 13.1 -> 10.3 ms.  One exponent per tile measured 950 us, 2410 us and 10.6
+// FP64 -> fixed point: Configuration 3 512^2 order 5, one step, 1235 -> 1000 us; the 1600 x 800 order-9 jet
+// residual 3564 -> 2375 us; 64 mixed problems 13.1 -> 10.4 ms.  One exponent per tile measured 950 us, 2410 us and 10.6
 // ms: it converts a value once, but cuts off the digits of values far below the tile's largest.
 // Flows without a front in both directions stay in FP64 to the bit: their strengths are differences of two
 // reconstructions that agree to rounding (1e-12 made of 1e-16 parts on a fine smooth grid), so
